@@ -331,7 +331,7 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
       mat_bytes += (block_dev_matrix_bytes(plan[i], c128) + 255) & ~(size_t)255;
     }
   bool any_tc = false;
-  for (const Block &b : plan) any_tc |= b.tc && !c128;
+  for (const Block &b : plan) any_tc |= b.tc;
   cudaError_t e;
   if (mat_bytes) {
     if (st->mats_copied) {

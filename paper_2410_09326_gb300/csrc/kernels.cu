@@ -355,15 +355,15 @@ const DevInfo &dev_info() {
 bool block_needs_dev_matrix(const Block &b, bool c128) {
   if (b.kind == BK_TILE || b.kind == BK_PHASE) return true;
   if (b.kind != BK_DENSE) return false;
-  if (b.tc && !c128) return true;
-  return b.k == 6 || (c128 && b.k == 5);
+  return b.tc || b.k == 6 || (c128 && b.k == 5);
 }
 
 size_t block_dev_matrix_bytes(const Block &b, bool c128) {
   if (!block_needs_dev_matrix(b, c128)) return 0;
   if (b.kind == BK_TILE) return tile_desc_bytes(b, c128);
   if (b.kind == BK_PHASE) return phase_desc_bytes(b, c128);
-  if (b.tc && !c128) return b.tc_tf32 ? tc_b_floats(b.k) * sizeof(float) : tc16_b_bytes(b.k);
+  if (b.tc && c128) return tc64_b_bytes(b.k);
+  if (b.tc) return b.tc_tf32 ? tc_b_floats(b.k) * sizeof(float) : tc16_b_bytes(b.k);
   return b.mat.size() * (c128 ? 16 : 8);
 }
 
@@ -376,8 +376,9 @@ void fill_dev_matrix(const Block &b, bool c128, void *host_out) {
     phase_fill_desc(b, c128, host_out);
     return;
   }
-  if (b.tc && !c128) {
-    if (b.tc_tf32) tc_build_b(b, (float *)host_out);
+  if (b.tc) {
+    if (c128) tc64_build_b(b, host_out);
+    else if (b.tc_tf32) tc_build_b(b, (float *)host_out);
     else tc16_build_b(b, host_out);
     return;
   }
@@ -397,7 +398,9 @@ cudaError_t launch_block_with_matrix(void *amps, int n, bool c128, const Block &
   if (threads <= 0) threads = 256;
   if (b.kind == BK_TILE) return run_tile(amps, n, c128, b, dev_mat, s);
   if (b.kind == BK_PHASE) return run_phase(amps, n, c128, b, dev_mat, s, shape);
-  if (b.kind == BK_DENSE && b.tc && !c128)
+  if (b.kind == BK_DENSE && b.tc && c128)
+    return run_dense_tc64((double2 *)amps, n, b, dev_mat, err, s, shape);
+  if (b.kind == BK_DENSE && b.tc)
     return b.tc_tf32 ? run_dense_tc((float2 *)amps, n, b, dev_mat, err, s, shape)
                      : run_dense_tc16((float2 *)amps, n, b, dev_mat, err, s, shape);
   if (c128) return run_block<double2>((double2 *)amps, n, b, dev_mat, s, threads);

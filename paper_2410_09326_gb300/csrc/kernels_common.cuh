@@ -213,6 +213,13 @@ void tc16_build_b(const Block &b, void *out);
 cudaError_t run_dense_tc16(float2 *a, int n, const Block &b, const void *dev_b, int *err, cudaStream_t s,
                            LaunchShape *shape);
 
+// complex128 blocks on the tensor cores (tc64.cu), k = 4, 5: dev_b holds
+// tc64_b_bytes(k) bytes written by tc64_build_b.
+size_t tc64_b_bytes(int k);
+void tc64_build_b(const Block &b, void *out);
+cudaError_t run_dense_tc64(double2 *a, int n, const Block &b, const void *dev_b, int *err, cudaStream_t s,
+                           LaunchShape *shape);
+
 // Cache-blocked passes (tile.cu): a BK_TILE block's descriptor (header,
 // member matrices and tables, member descriptors) lives in device memory.
 size_t tile_desc_bytes(const Block &b, bool c128);

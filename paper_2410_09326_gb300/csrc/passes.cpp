@@ -921,13 +921,14 @@ qs_status build_plan(int n, const qs_gate *gates, size_t n_gates, uint64_t flags
   }
   const bool tf32 = opts.tc_precision == 1;
   for (Block &b : plan) {
-    b.tc = (flags & QS_TC) && b.kind == BK_DENSE && b.k >= 4 && b.k <= (tf32 ? 5 : 6);
-    b.tc_tf32 = b.tc && tf32;
+    // complex128 blocks run on FP16 digit planes (tc64.cu), 4 and 5 targets
+    b.tc = (flags & QS_TC) && b.kind == BK_DENSE && b.k >= 4 && b.k <= (tf32 || c128 ? 5 : 6);
+    b.tc_tf32 = b.tc && tf32 && !c128;
     b.shuffles = opts.no_shuffles == 0;
     // lane-exchange gathers where they measured faster (tc_exchange_pays),
     // or everywhere the layout allows with tc_exchange = 2
     TcXLayout xl;
-    b.tc_xg = b.tc && !tf32 && opts.tc_exchange != 1 && (opts.tc_exchange == 2 || tc_exchange_pays(b)) &&
+    b.tc_xg = b.tc && !tf32 && !c128 && opts.tc_exchange != 1 && (opts.tc_exchange == 2 || tc_exchange_pays(b)) &&
               tc_exchange_layout(n, b, xl);
     b.withhold_commit = b.tc && opts.test_wait_timeout != 0;
     b.tc_max_ctas = (b.tc || b.kind == BK_PHASE) ? opts.tc_max_ctas : 0;
