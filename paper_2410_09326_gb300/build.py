@@ -62,7 +62,7 @@ def _compile(src, verbose):
             cmd.insert(1, "-Xptxas=-v")
     else:
         # -fcx-limited-range: plain complex products (gate entries are finite)
-        cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-fcx-limited-range", "-pthread", "-Wall",
+        cmd = ["g++", "-O3", "-std=c++17", "-fPIC", "-fcx-limited-range", "-pthread", "-Wall",
                "-Wno-unused-function",
                "-I", INC, "-I", SRC, "-I", os.path.join(cuda, "include"), "-c", path, "-o", obj]
     r = subprocess.run(cmd, capture_output=True, text=True)

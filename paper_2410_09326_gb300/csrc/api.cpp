@@ -361,7 +361,7 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
       st->d_mats = dm;
       st->mats_cap = mat_bytes;
     }
-    parallel_blocks(plan.size(), [&](size_t i) {
+    parallel_blocks(plan.size(), 1e-3 * (double)mat_bytes, [&](size_t i) {
       if (mat_off[i] != (size_t)-1) fill_dev_matrix(plan[i], c128, (unsigned char *)st->h_mats + mat_off[i]);
     });
     e = cudaMemcpyAsync(st->d_mats, st->h_mats, mat_bytes, cudaMemcpyHostToDevice, st->stream);

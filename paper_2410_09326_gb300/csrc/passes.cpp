@@ -22,8 +22,8 @@ namespace {
 
 constexpr double kEps = 1e-14;
 
-bool is_one(cd z) { return std::abs(z - cd(1, 0)) <= kEps; }
-bool is_zero(cd z) { return std::abs(z) <= kEps; }
+bool is_one(cd z) { return std::norm(z - cd(1, 0)) <= kEps * kEps; }
+bool is_zero(cd z) { return std::norm(z) <= kEps * kEps; }
 
 int popcount64(uint64_t x) { return __builtin_popcountll(x); }
 
@@ -34,53 +34,80 @@ int pos_of(const int *qs, int w, int q) {
   return -1;
 }
 
-// Applies a gate's full matrix G (on local positions pos[0..m)) from the left
-// to every column of the block matrix M (2^w x 2^w, row-major).
-void left_multiply(std::vector<cd> &M, int w, const std::vector<cd> &G, const int *pos, int m) {
-  const int d = 1 << w, dg = 1 << m;
-  int gmask = 0;
+// A block's product under construction: 2^w x 2^w, real and imaginary parts
+// apart, so that the loops over a row's columns vectorise.
+struct Product {
+  int d;
+  std::vector<double> re, im, tre, tim;
+  explicit Product(int w) : d(1 << w), re((size_t)d * d, 0.0), im((size_t)d * d, 0.0), tre(8 * d), tim(8 * d) {
+    for (int i = 0; i < d; i++) re[(size_t)i * d + i] = 1;
+  }
+  cd at(int r, int c) const { return cd(re[(size_t)r * d + c], im[(size_t)r * d + c]); }
+};
+
+// Applies a gate's full matrix G (on local positions pos[0..m), m <= 3) from
+// the left: row combinations, zero entries and unchanged rows skipped.
+void left_multiply(Product &M, const std::vector<cd> &G, const int *pos, int m) {
+  const int d = M.d, dg = 1 << m;
+  int gmask = 0, off[8];
   for (int j = 0; j < m; j++) gmask |= 1 << pos[j];
-  std::vector<cd> v(dg), r(dg);
-  for (int col = 0; col < d; col++) {
-    for (int base = 0; base < d; base++) {
-      if (base & gmask) continue;
-      for (int l = 0; l < dg; l++) {
-        int idx = base;
-        for (int j = 0; j < m; j++)
-          if ((l >> j) & 1) idx |= 1 << pos[j];
-        v[l] = M[(size_t)idx * d + col];
+  bool same[8];
+  for (int l = 0; l < dg; l++) {
+    off[l] = 0;
+    for (int j = 0; j < m; j++)
+      if ((l >> j) & 1) off[l] |= 1 << pos[j];
+    same[l] = true;
+    for (int b = 0; b < dg; b++) same[l] = same[l] && G[(size_t)l * dg + b] == cd(b == l ? 1 : 0, 0);
+  }
+  for (int base = 0; base < d; base++) {
+    if (base & gmask) continue;
+    for (int a = 0; a < dg; a++) {
+      if (same[a]) continue;
+      double *tr = M.tre.data() + (size_t)a * d, *ti = M.tim.data() + (size_t)a * d;
+      bool first = true;
+      for (int b = 0; b < dg; b++) {
+        const double gr = G[(size_t)a * dg + b].real(), gi = G[(size_t)a * dg + b].imag();
+        if (gr == 0 && gi == 0) continue;
+        const double *xr = M.re.data() + (size_t)(base | off[b]) * d, *xi = M.im.data() + (size_t)(base | off[b]) * d;
+        if (first)
+          for (int c = 0; c < d; c++) {
+            tr[c] = gr * xr[c] - gi * xi[c];
+            ti[c] = gr * xi[c] + gi * xr[c];
+          }
+        else
+          for (int c = 0; c < d; c++) {
+            tr[c] += gr * xr[c] - gi * xi[c];
+            ti[c] += gr * xi[c] + gi * xr[c];
+          }
+        first = false;
       }
-      for (int a = 0; a < dg; a++) {
-        cd acc = 0;
-        for (int b = 0; b < dg; b++) acc += G[(size_t)a * dg + b] * v[b];
-        r[a] = acc;
-      }
-      for (int l = 0; l < dg; l++) {
-        int idx = base;
-        for (int j = 0; j < m; j++)
-          if ((l >> j) & 1) idx |= 1 << pos[j];
-        M[(size_t)idx * d + col] = r[l];
-      }
+    }
+    for (int a = 0; a < dg; a++) {
+      if (same[a]) continue;
+      std::memcpy(M.re.data() + (size_t)(base | off[a]) * d, M.tre.data() + (size_t)a * d, sizeof(double) * d);
+      std::memcpy(M.im.data() + (size_t)(base | off[a]) * d, M.tim.data() + (size_t)a * d, sizeof(double) * d);
     }
   }
 }
 
-// Runs f(0..n) on up to 16 host threads when the work is large enough to pay
-// for them (block products are independent once the grouping is fixed).
-template <typename F> void parallel_for(size_t n, F f) {
-  unsigned nt = std::min(16u, std::max(1u, std::thread::hardware_concurrency()));
-  if (n < 16 || nt <= 1) {
+// Runs f(0..n) on as many host threads (up to 16) as work_us, the estimated
+// microseconds of all the calls together, pays for: starting and joining a
+// thread costs about as much as 50 us of work, so a thread is given 100.
+template <typename F> void parallel_for(size_t n, double work_us, F f) {
+  const unsigned most = std::min(16u, std::max(1u, std::thread::hardware_concurrency()));
+  const size_t nt = std::min<size_t>({most, n, (size_t)(work_us / 100) + 1});
+  if (nt <= 1) {
     for (size_t i = 0; i < n; i++) f(i);
     return;
   }
-  if (nt > n / 4) nt = (unsigned)std::max<size_t>(1, n / 4);
   std::atomic<size_t> next{0};
+  auto work = [&] {
+    for (size_t i; (i = next.fetch_add(1)) < n;) f(i);
+  };
   std::vector<std::thread> th;
-  th.reserve(nt);
-  for (unsigned t = 0; t < nt; t++)
-    th.emplace_back([&] {
-      for (size_t i; (i = next.fetch_add(1)) < n;) f(i);
-    });
+  th.reserve(nt - 1);
+  for (size_t t = 1; t < nt; t++) th.emplace_back(work);
+  work();
   for (auto &x : th) x.join();
 }
 
@@ -154,10 +181,12 @@ void greedy_groups(const std::vector<qs_gate> &pg, const std::vector<int> &idx, 
 // whose roll-out ends with the fewest blocks -- then the narrowest recent
 // blocks -- is kept; ties keep the earliest candidate (first fit). Placement
 // obeys the same commutation rule and width limits as greedy_groups.
-// limit(all_diag_block_and_gate) is the width bound.
+// limit(all_diag_block_and_gate) is the width bound. With free_joins a gate
+// whose first candidate needs no further qubit for it joins that one without
+// roll-outs: it widens nothing and holds later gates back the least.
 template <typename Limit>
 void lookahead_groups(const std::vector<qs_gate> &pg, const std::vector<int> &idx, std::vector<Pending> &groups,
-                      Limit limit, int horizon, int tail_blocks = 6) {
+                      Limit limit, int horizon, int tail_blocks, bool free_joins) {
   struct LG {
     uint64_t qmask;
     bool all_diag;
@@ -211,7 +240,8 @@ void lookahead_groups(const std::vector<qs_gate> &pg, const std::vector<int> &id
       if (fits(G[b], x)) cand[nc++] = b;
     cand[nc++] = (int)G.size();
     int ch = cand[0];
-    if (nc > 1 && horizon > 0) {
+    const bool join = free_joins && nc > 1 && (x.gmask & ~G[ch].qmask) == 0 && (x.gdiag || !G[ch].all_diag);
+    if (nc > 1 && horizon > 0 && !join) {
       long best_blocks = -1, best_tail = 0;
       for (int c = 0; c < nc; c++) {
         G2 = G;
@@ -219,7 +249,8 @@ void lookahead_groups(const std::vector<qs_gate> &pg, const std::vector<int> &id
         std::memcpy(ln2, ln, sizeof(ln));
         place(G2, la2, ln2, x, cand[c]);
         const int end = std::min(N, i + 1 + horizon);
-        for (int j = i + 1; j < end; j++) {
+        // (the block count only grows: a roll-out past the best one's is lost)
+        for (int j = i + 1; j < end && (best_blocks < 0 || (long)G2.size() <= best_blocks); j++) {
           const GI &y = info[j];
           int b = std::max(lower_of(y, la2, ln2), 0);
           while (b < (int)G2.size() && !fits(G2[b], y)) b++;
@@ -406,14 +437,13 @@ bool finish_block(const std::vector<qs_gate> &pg, const Pending &p, bool allow_p
   }
   // dense product over the w qubits
   const int d = 1 << w;
-  std::vector<cd> M((size_t)d * d, cd(0, 0));
-  for (int i = 0; i < d; i++) M[(size_t)i * d + i] = 1;
+  Product M(w);
   for (int gi : p.members) {
     const qs_gate &g = pg[gi];
     gate_full_matrix(g, G);
     int pos[8];
     for (int j = 0; j < g.nq; j++) pos[j] = pos_of(qs, w, g.q[j]);
-    left_multiply(M, w, G, pos, g.nq);
+    left_multiply(M, G, pos, g.nq);
   }
   // control detection: block-diagonal in bit j with identity on the 0 half
   uint64_t cmask = 0;
@@ -422,7 +452,7 @@ bool finish_block(const std::vector<qs_gate> &pg, const Pending &p, bool allow_p
     bool ctrl = true;
     for (int r = 0; r < d && ctrl; r++)
       for (int c = 0; c < d && ctrl; c++) {
-        cd z = M[(size_t)r * d + c];
+        cd z = M.at(r, c);
         int br = (r >> j) & 1, bc = (c >> j) & 1;
         if (br != bc) { if (!is_zero(z)) ctrl = false; }
         else if (br == 0) { if (r == c ? !is_one(z) : !is_zero(z)) ctrl = false; }
@@ -442,13 +472,15 @@ bool finish_block(const std::vector<qs_gate> &pg, const Pending &p, bool allow_p
       if ((l2 >> j) & 1) l |= 1 << keep[j];
     return l;
   };
-  for (int r = 0; r < dk; r++)
+  for (int r = 0; r < dk; r++) {
+    const int er = expand(r);
     for (int c = 0; c < dk; c++) {
-      cd z = M[(size_t)expand(r) * d + expand(c)];
+      cd z = M.at(er, nk == w ? c : expand(c));
       R[(size_t)r * dk + c] = z;
-      if (r != c && !is_zero(z)) diag = false, identity = false;
-      if (r == c && !is_one(z)) identity = false;
+      if (diag && r != c && !is_zero(z)) diag = false, identity = false;
+      if (identity && r == c && !is_one(z)) identity = false;
     }
+  }
   if (identity) return false;
   out.cmask = cmask;
   out.nctrl = popcount64(cmask);
@@ -465,6 +497,18 @@ bool finish_block(const std::vector<qs_gate> &pg, const Pending &p, bool allow_p
   return true;
 }
 
+// Estimated host time of the groups' products: a gate on a w-qubit dense
+// block updates 4^w entries at about a nanosecond each, on a diagonal one 2^w.
+double products_us(const std::vector<Pending> &groups) {
+  double us = 0;
+  for (const Pending &p : groups) {
+    const int w = popcount64(p.qmask);
+    us += 0.3 + (double)p.members.size() * (0.1 + 1e-3 * (p.all_diag ? (w <= QS_MAX_DIAG ? 4.0 * (1 << w) : 100.0)
+                                                                     : std::ldexp(1.0, 2 * w)));
+  }
+  return us;
+}
+
 void push_exchanges(const std::vector<std::pair<int, int>> &reloc, std::vector<Block> &plan) {
   for (auto &pr : reloc) {  // the exchanges run first
     Block b;
@@ -477,6 +521,9 @@ void push_exchanges(const std::vector<std::pair<int, int>> &reloc, std::vector<B
     plan.push_back(std::move(b));
   }
 }
+
+constexpr int kSearchBits = 23;      // narrowest complex64 state whose fusion is searched
+constexpr int kFullSearchBits = 27;  // and without free joins too
 
 constexpr int kTileMaxOps = 64;     // member blocks of one tile pass
 constexpr int kTilePool = 2048;     // matrix + phase-table entries of one tile pass
@@ -508,7 +555,7 @@ qs_status tile_plan(int n, const std::vector<qs_gate> &pg, const std::vector<int
     tmask[pi] = t;
   }
   std::vector<uint64_t> cl(pg.size(), 0);
-  parallel_for(pg.size(), [&](size_t i) { cl[i] = ctrl_like_mask(pg[i]); });
+  parallel_for(pg.size(), 0.1 * (double)pg.size(), [&](size_t i) { cl[i] = ctrl_like_mask(pg[i]); });
   // member blocks of every pass
   std::vector<Pending> subs;
   std::vector<int> sub_pass;
@@ -537,7 +584,7 @@ qs_status tile_plan(int n, const std::vector<qs_gate> &pg, const std::vector<int
   }
   std::vector<Block> done(subs.size());
   std::vector<char> keep(subs.size(), 0);
-  parallel_for(subs.size(), [&](size_t i) { keep[i] = finish_block(pg, subs[i], false, done[i]) ? 1 : 0; });
+  parallel_for(subs.size(), products_us(subs), [&](size_t i) { keep[i] = finish_block(pg, subs[i], false, done[i]) ? 1 : 0; });
   (void)err;
   size_t si = 0;
   for (size_t pi = 0; pi < passes.size(); pi++) {
@@ -596,8 +643,8 @@ qs_status tile_plan(int n, const std::vector<qs_gate> &pg, const std::vector<int
 // Fusion and classification of the physical gates pg[idx...] (one segment
 // of the circuit between global-tier exchanges); appends the blocks.
 qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<int> &all, uint64_t flags,
-                       const qs_opts &opts, int D, int K, bool c128, bool allow_phase, std::vector<Block> &plan,
-                       std::string &err) {
+                       const qs_opts &opts, int D, int K, bool c128, bool allow_phase, bool repeated,
+                       std::vector<Block> &plan, std::string &err) {
   const bool fuse = flags & QS_FUSE;
   const bool dfuse = flags & QS_DIAG;
   std::vector<Pending> groups;
@@ -623,33 +670,50 @@ qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<
     const bool phase_ok = dfuse && allow_phase && n > QS_MAX_DIAG;
     const int dlimit = phase_ok ? 64 : D;
     auto limit = [&](bool nd) { return nd ? (dfuse ? dlimit : std::max(K, 1)) : K; };
-    if (opts.fuse_lookahead > 0) {
-      // the roll-out heuristic usually saves blocks but is not guaranteed
-      // to, and its best horizon and tie-break vary: plain first fit and
-      // roll-outs of L, 4L/3 and 5L/3 gates (ties broken by the width of the
-      // last 6 or 12 blocks) run side by side on host threads, and the
-      // grouping with the fewest blocks is launched (earliest on a tie)
-      constexpr int kVariants = 6;
-      std::vector<Pending> alt[kVariants];
-      const int L = opts.fuse_lookahead;
-      const int horizons[kVariants] = {0, L, L, L + L / 3, L + L / 3, L + 2 * L / 3};
-      const int tails[kVariants] = {0, 6, 12, 6, 12, 6};
-      run_tasks(kVariants, [&](size_t v) {
-        if (v == 0)
-          greedy_groups(pg, all, alt[0], [&](const Pending &p, int, uint64_t gmask, uint64_t, bool gdiag) {
-            return popcount64(p.qmask | gmask) <= limit(p.all_diag && gdiag);
-          });
-        else
-          lookahead_groups(pg, all, alt[v], limit, horizons[v], tails[v]);
+    auto first_fit = [&](std::vector<Pending> &g) {
+      greedy_groups(pg, all, g, [&](const Pending &p, int, uint64_t gmask, uint64_t, bool gdiag) {
+        return popcount64(p.qmask | gmask) <= limit(p.all_diag && gdiag);
       });
-      int best = 0;
-      for (int v = 1; v < kVariants; v++)
+    };
+    // The search saves one block in six on layered circuits, so it has to
+    // cost less than that share of the passes. Roll-outs with free joins cost
+    // about 1 us of host time per gate, and a gate about a twelfth of a pass:
+    // they pay from 23 qubits on (20 us a pass in complex64; complex128
+    // passes take five times as long and pay from 22 on), or where a plan is
+    // run again and again (a batch). Without free joins they cost 5 us per
+    // gate and sometimes save a few blocks more at 6 targets (98 instead of
+    // 107 for the 30-qubit random circuit): from 27 qubits on (25).
+    const int wide = n + (c128 ? 1 : 0);
+    if (opts.fuse_lookahead > 0 && (wide >= kSearchBits || repeated)) {
+      // no horizon or tie-break (by the width of the last 6 or 12 blocks) is
+      // best on every circuit: first fit and several roll-outs run side by
+      // side on host threads, and the grouping with the fewest blocks is
+      // launched (the earliest on a tie)
+      struct Variant {
+        int horizon, tail;
+        bool free_joins;
+      };
+      const int L = opts.fuse_lookahead;
+      const Variant variants[] = {{0, 0, false},          {L, 6, true},       {L, 12, true},
+                                  {L + L / 3, 6, true},   {L, 6, false},      {L, 12, false},
+                                  {L + L / 3, 6, false},  {L + L / 3, 12, false}, {L + 2 * L / 3, 6, false}};
+      const size_t count = n + (c128 ? 2 : 0) >= kFullSearchBits ? 9 : 4;
+      std::vector<std::vector<Pending>> alt(count);
+      auto one = [&](size_t v) {
+        if (v == 0) first_fit(alt[0]);
+        else lookahead_groups(pg, all, alt[v], limit, variants[v].horizon, variants[v].tail, variants[v].free_joins);
+      };
+      if (repeated) {  // many circuits are planned one after the other: threads would cost more than they save
+        for (size_t v = 0; v < count; v++) one(v);
+      } else {
+        run_tasks(count, one);
+      }
+      size_t best = 0;
+      for (size_t v = 1; v < count; v++)
         if (alt[v].size() < alt[best].size()) best = v;
       groups.swap(alt[best]);
     } else {
-      greedy_groups(pg, all, groups, [&](const Pending &p, int, uint64_t gmask, uint64_t, bool gdiag) {
-        return popcount64(p.qmask | gmask) <= limit(p.all_diag && gdiag);
-      });
+      first_fit(groups);
     }
   }
 
@@ -657,7 +721,7 @@ qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<
   std::vector<Block> done(groups.size());
   std::vector<char> keep(groups.size(), 0);
   const bool phase_ok = dfuse && allow_phase && n > QS_MAX_DIAG;
-  parallel_for(groups.size(), [&](size_t i) {
+  parallel_for(groups.size(), repeated ? 0 : products_us(groups), [&](size_t i) {
     if (!groups[i].members.empty()) keep[i] = finish_block(pg, groups[i], true, done[i], D, phase_ok) ? 1 : 0;
   });
   for (size_t i = 0; i < groups.size(); i++)
@@ -667,7 +731,7 @@ qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<
 
 }  // namespace
 
-void parallel_blocks(size_t n, const std::function<void(size_t)> &f) { parallel_for(n, f); }
+void parallel_blocks(size_t n, double work_us, const std::function<void(size_t)> &f) { parallel_for(n, work_us, f); }
 
 int tile_bits_of(const qs_opts &o, bool c128) {
   if (o.tile_bits > 0) return std::min(o.tile_bits, c128 ? kMaxTileBits - 1 : kMaxTileBits);
@@ -704,7 +768,7 @@ double block_bytes(const Block &b, int n, int amp_bytes) {
 
 qs_status build_plan(int n, const qs_gate *gates, size_t n_gates, uint64_t flags,
                      const qs_opts &opts, int8_t *perm, std::vector<Block> &plan,
-                     PlanStats &stats, std::string &err, bool c128, bool allow_phase) {
+                     PlanStats &stats, std::string &err, bool c128, bool allow_phase, bool repeated) {
   plan.clear();
   stats = PlanStats();
   stats.gates_in = (int)n_gates;
@@ -905,7 +969,7 @@ qs_status build_plan(int n, const qs_gate *gates, size_t n_gates, uint64_t flags
     const size_t seg_end = sgi < cuts.size() ? cuts[sgi] : pg.size();
     std::vector<int> idx;
     for (size_t i = seg_begin; i < seg_end; i++) idx.push_back((int)i);
-    qs_status st = plan_segment(n, pg, idx, flags, opts, D, K, c128, allow_phase, plan, err);
+    qs_status st = plan_segment(n, pg, idx, flags, opts, D, K, c128, allow_phase, repeated, plan, err);
     if (st != QS_OK) return st;
     if (sgi < cuts.size()) {
       Block b;

@@ -126,9 +126,12 @@ struct PlanStats {
 // state's logical->physical map, updated in place for absorbed SWAPs.
 // Returns QS_OK or QS_EINVAL (message in err).
 // c128 selects the amplitude size the default tile width is computed for.
+// repeated: the plan will run many times, so that fusion is searched at any
+// width.
 qs_status build_plan(int n, const qs_gate *gates, size_t n_gates, uint64_t flags,
                      const qs_opts &opts, int8_t *perm, std::vector<Block> &plan,
-                     PlanStats &stats, std::string &err, bool c128 = false, bool allow_phase = true);
+                     PlanStats &stats, std::string &err, bool c128 = false, bool allow_phase = true,
+                     bool repeated = false);
 
 // Tile width QS_TILE uses for these options and amplitude type.
 int tile_bits_of(const qs_opts &o, bool c128);
@@ -142,8 +145,8 @@ void fill_record(const Block &b, int index, int n, int amp_bytes, qs_block_recor
 // Cost-model features of a block record (pgo.cpp).
 void record_features(const qs_block_record &r, int n, bool c128, float *f);
 
-// f(0..n) on a few host threads (passes.cpp).
-void parallel_blocks(size_t n, const std::function<void(size_t)> &f);
+// f(0..n) on as many host threads as the estimated work pays for (passes.cpp).
+void parallel_blocks(size_t n, double work_us, const std::function<void(size_t)> &f);
 
 // Rotation folding + peephole cancellation (fold.cpp): an equivalent gate
 // list (exact, global phase included).
