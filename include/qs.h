@@ -245,7 +245,8 @@ typedef struct {
   double t_start_ms; /* start relative to the first block (QS_PROFILE), else -1 */
   double ms;         /* device time (QS_PROFILE), else -1 */
   int64_t tiles;     /* blocks of an apply call: tensor-core blocks, tiles of 128 groups;
-                        phase polynomials, chunks of 1024 amplitudes; else 0 */
+                        phase polynomials, chunks of 1024 amplitudes; else 0 (also where a
+                        narrow state's blocks share one launch) */
   int32_t ctas;      /* the same blocks: CTAs launched (each loops over tiles ctas apart;
                         each of a phase CTA's 8 warps over chunks 8 ctas apart); else 0 */
   int32_t reserved;

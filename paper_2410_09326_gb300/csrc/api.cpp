@@ -308,7 +308,7 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
     // a first call has no measurements yet: profile it so the next one has
     flags = f | QS_PROFILE;
   } else if (flags & QS_PGO_RULES) {
-    flags = rules_select(st->n, gates, n_gates, o, flags);
+    flags = rules_select(st->n, st->dtype == QS_C128, gates, n_gates, o, flags);
   }
 
   std::vector<Block> plan;
@@ -322,11 +322,16 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
 
   const bool c128 = st->dtype == QS_C128;
   const int ab = amp_bytes(st);
+  const bool prof = flags & QS_PROFILE;
+  // narrow states: every block in one launch (not for plain per-gate runs,
+  // nor where each block is timed)
+  const bool resident = !c128 && !prof && (flags & (QS_FUSE | QS_DIAG)) && o.threads == 0 && o.tc_max_ctas == 0 &&
+                        resident_applies(plan, st->n);
   // matrices of wide dense blocks: one pinned staging buffer, one copy
   size_t mat_bytes = 0;
   std::vector<size_t> mat_off(plan.size(), (size_t)-1);
   for (size_t i = 0; i < plan.size(); i++)
-    if (block_needs_dev_matrix(plan[i], c128)) {
+    if (!resident && block_needs_dev_matrix(plan[i], c128)) {
       mat_off[i] = mat_bytes;
       mat_bytes += (block_dev_matrix_bytes(plan[i], c128) + 255) & ~(size_t)255;
     }
@@ -375,7 +380,6 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
     if (e == cudaSuccess) e = cudaMemsetAsync(st->d_err, 0, sizeof(int), st->stream);
     if (e != cudaSuccess) return fail(QS_ENOMEM, "error word allocation failed");
   }
-  const bool prof = flags & QS_PROFILE;
   if (prof) {
     while (st->events.size() < plan.size() + 1) {
       cudaEvent_t ev;
@@ -390,12 +394,18 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
   st->rec_class.clear();
   st->recs.reserve(plan.size());
   st->h2d_bytes = 0;
+  if (resident) {
+    e = run_resident(st->amps, st->n, plan, st->stream);
+    if (e != cudaSuccess) return cuda_fail(st, e, "qs_apply_circuit launch");
+  }
   for (size_t i = 0; i < plan.size(); i++) {
     const Block &b = plan[i];
     const void *dm = mat_off[i] == (size_t)-1 ? nullptr : (const unsigned char *)st->d_mats + mat_off[i];
     LaunchShape shape;
-    e = launch_block_with_matrix(st->amps, st->n, c128, b, dm, st->d_err, st->stream, o.threads, &shape);
-    if (e != cudaSuccess) return cuda_fail(st, e, "qs_apply_circuit launch");
+    if (!resident) {
+      e = launch_block_with_matrix(st->amps, st->n, c128, b, dm, st->d_err, st->stream, o.threads, &shape);
+      if (e != cudaSuccess) return cuda_fail(st, e, "qs_apply_circuit launch");
+    }
     if (prof) {
       e = cudaEventRecord(st->events[i + 1], st->stream);
       if (e != cudaSuccess) return cuda_fail(st, e, "qs_apply_circuit");
@@ -577,7 +587,7 @@ qs_status qs_plan(int n, const qs_gate *gates, size_t n_gates, uint64_t flags, c
   qs_opts o;
   if (opts) o = *opts;
   else qs_default_opts(&o);
-  if (flags & QS_PGO_RULES) flags = rules_select(n, gates, n_gates, o, flags);
+  if (flags & QS_PGO_RULES) flags = rules_select(n, false, gates, n_gates, o, flags);
   std::vector<Block> plan;
   PlanStats stats;
   std::string err;

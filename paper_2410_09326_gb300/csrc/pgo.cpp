@@ -80,7 +80,7 @@ double predict_plan_ms(const std::vector<Block> &plan, int n, int amp_bytes, con
 
 // Rule-based activator (Sec. III-A "PGO compilation flow", Sec. III-D):
 // one decision per optimisation from the counters of the circuit at hand.
-uint64_t rules_select(int n, const qs_gate *gates, size_t n_gates, const qs_opts &o, uint64_t base) {
+uint64_t rules_select(int n, bool c128, const qs_gate *gates, size_t n_gates, const qs_opts &o, uint64_t base) {
   int run[QS_MAX_QUBITS] = {0}, max_run = 0;
   int64_t swaps = 0, two_q_low = 0, t_count = 0, dense = 0;
   for (size_t i = 0; i < n_gates; i++) {
@@ -97,7 +97,6 @@ uint64_t rules_select(int n, const qs_gate *gates, size_t n_gates, const qs_opts
         two_q_low++;
     }
   }
-  (void)n;
   uint64_t f = base & ~(uint64_t)(QS_VSWAP | QS_FUSE | QS_DIAG | QS_FOLD | QS_RELOCATE | QS_TILE | (15ull << 16));
   // rotation folding: T gates above the threshold share of all gates
   if (n_gates && (double)t_count / (double)n_gates > o.t_ratio) f |= QS_FOLD;
@@ -110,7 +109,10 @@ uint64_t rules_select(int n, const qs_gate *gates, size_t n_gates, const qs_opts
   // merging: a run of consecutive one-qubit gates above the threshold, or
   // (GPU reading) any circuit with more than one gate, since each fused gate
   // saves a full pass over the state
-  if (max_run > o.merge_run || n_gates > 1) f |= QS_FUSE | QS_FUSE_K(5) | QS_DIAG | QS_TC;
+  // Narrow complex64 states take 3-qubit blocks, which one launch applies in
+  // shared memory (resident.cu): a wider block saves no pass over HBM there.
+  if (max_run > o.merge_run || n_gates > 1)
+    f |= !c128 && n <= kResidentBits ? (QS_FUSE | QS_FUSE_K(3) | QS_DIAG) : (QS_FUSE | QS_FUSE_K(5) | QS_DIAG | QS_TC);
   (void)dense;
   return f;
 }

@@ -153,7 +153,7 @@ void parallel_blocks(size_t n, double work_us, const std::function<void(size_t)>
 std::vector<qs_gate> fold_rotations(int n, const qs_gate *in, size_t n_in);
 
 // Profile-guided selection (pgo.cpp).
-uint64_t rules_select(int n, const qs_gate *gates, size_t n_gates, const qs_opts &o, uint64_t base);
+uint64_t rules_select(int n, bool c128, const qs_gate *gates, size_t n_gates, const qs_opts &o, uint64_t base);
 int block_class(const Block &b);
 double predict_plan_ms(const std::vector<Block> &plan, int n, int amp_bytes, const qs_class_table *t,
                        double peak_gbs);
@@ -200,6 +200,12 @@ size_t block_param_bytes(const Block &b, bool c128);
 // shape (may be null) receives a tensor-core launch's tiles and CTAs.
 cudaError_t launch_block_with_matrix(void *amps, int n, bool c128, const Block &b, const void *dev_mat,
                                      int *err, cudaStream_t s, int threads, LaunchShape *shape = nullptr);
+// Narrow complex64 states (resident.cu): whether the whole plan can run in
+// shared memory, and the launches that do it (as few as its records fit the
+// kernel parameters).
+constexpr int kResidentBits = 13;
+bool resident_applies(const std::vector<Block> &plan, int n);
+cudaError_t run_resident(void *amps, int n, const std::vector<Block> &plan, cudaStream_t s);
 cudaError_t launch_permute(void *amps, int n, bool c128, int a, int b, cudaStream_t s);
 cudaError_t launch_set_basis(void *amps, int n, bool c128, uint64_t idx, cudaStream_t s);
 
