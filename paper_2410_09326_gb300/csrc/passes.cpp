@@ -536,8 +536,10 @@ constexpr int kTilePool = 2048;     // matrix + phase-table entries of one tile 
 // into shared memory, applies the pass's member blocks there, and stores it.
 // Inside a pass the gates are fused again, at most tile_k qubits wide; a
 // qubit outside the tile may only be a control or sit in a diagonal block.
+// repeated (batches): a pass with one member stays a pass, and diagonal runs
+// become phase polynomials of any width.
 qs_status tile_plan(int n, const std::vector<qs_gate> &pg, const std::vector<int> &all, const qs_opts &opts,
-                    bool c128, std::vector<Block> &out, std::string &err) {
+                    bool c128, bool repeated, std::vector<Block> &out, std::string &err) {
   const int m = tile_bits_of(opts, c128);
   const int kin = tile_k_of(opts);
   const int D = std::max(1, std::min(opts.diag_max, QS_MAX_DIAG));
@@ -555,7 +557,7 @@ qs_status tile_plan(int n, const std::vector<qs_gate> &pg, const std::vector<int
     tmask[pi] = t;
   }
   std::vector<uint64_t> cl(pg.size(), 0);
-  parallel_for(pg.size(), 0.1 * (double)pg.size(), [&](size_t i) { cl[i] = ctrl_like_mask(pg[i]); });
+  parallel_for(pg.size(), repeated ? 0 : 0.1 * (double)pg.size(), [&](size_t i) { cl[i] = ctrl_like_mask(pg[i]); });
   // member blocks of every pass
   std::vector<Pending> subs;
   std::vector<int> sub_pass;
@@ -566,7 +568,7 @@ qs_status tile_plan(int n, const std::vector<qs_gate> &pg, const std::vector<int
         pg, passes[pi].members, sg,
         [&](const Pending &p, int i, uint64_t gmask, uint64_t, bool gdiag) {
           const int width = popcount64(p.qmask | gmask);
-          if (p.all_diag && gdiag) return width <= D;
+          if (p.all_diag && gdiag) return repeated || width <= D;
           // a non-diagonal block may reach outside the tile only through
           // qubits that are controls of every member: then they are
           // detected as controls of the product
@@ -584,7 +586,9 @@ qs_status tile_plan(int n, const std::vector<qs_gate> &pg, const std::vector<int
   }
   std::vector<Block> done(subs.size());
   std::vector<char> keep(subs.size(), 0);
-  parallel_for(subs.size(), products_us(subs), [&](size_t i) { keep[i] = finish_block(pg, subs[i], false, done[i]) ? 1 : 0; });
+  parallel_for(subs.size(), repeated ? 0 : products_us(subs), [&](size_t i) {
+    keep[i] = finish_block(pg, subs[i], false, done[i], repeated ? 0 : QS_MAX_DIAG, repeated) ? 1 : 0;
+  });
   (void)err;
   size_t si = 0;
   for (size_t pi = 0; pi < passes.size(); pi++) {
@@ -597,9 +601,15 @@ qs_status tile_plan(int n, const std::vector<qs_gate> &pg, const std::vector<int
       if (b.kind == BK_DENSE) {
         ok = ok && b.k <= 4;
         for (int j = 0; j < b.k; j++) ok = ok && ((T >> b.q[j]) & 1);
-      } else if (b.kind != BK_DIAG) {
+      } else if (b.kind == BK_DIAG) {
+        for (int j = 0; j < b.k && repeated; j++) ok = ok && ((T >> b.q[j]) & 1);
+      } else if (b.kind != BK_PHASE) {
         ok = false;
       }
+    }
+    if (!ok && repeated) {
+      err = "tile pass with a member outside its tile";
+      return QS_EUNSUPPORTED;
     }
     if (!ok) {  // cannot happen by construction; the members stay valid alone
       for (Block &b : members) out.push_back(std::move(b));
@@ -612,12 +622,12 @@ qs_status tile_plan(int n, const std::vector<qs_gate> &pg, const std::vector<int
       int pool = 0;
       while (b1 < members.size() && (int)(b1 - b0) < kTileMaxOps) {
         const Block &b = members[b1];
-        const int ent = b.kind == BK_DENSE ? (1 << (2 * b.k)) : (1 << b.k);
+        const int ent = b.kind == BK_DENSE ? (1 << (2 * b.k)) : (b.kind == BK_PHASE ? (n + 4) * (n + 2) / 2 : 1 << b.k);
         if (b1 > b0 && pool + ent > kTilePool) break;
         pool += ent;
         b1++;
       }
-      if (b1 - b0 == 1) {
+      if (b1 - b0 == 1 && !repeated) {
         out.push_back(std::move(members[b0]));
       } else {
         Block t;
@@ -651,7 +661,7 @@ qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<
   const bool tiled = (flags & QS_TILE) && n > tile_bits_of(opts, c128);
   if (tiled) {
     std::vector<Block> tplan;
-    qs_status ts = tile_plan(n, pg, all, opts, c128, tplan, err);
+    qs_status ts = tile_plan(n, pg, all, opts, c128, repeated, tplan, err);
     if (ts != QS_OK) return ts;
     for (Block &b : tplan) plan.push_back(std::move(b));
     return QS_OK;
