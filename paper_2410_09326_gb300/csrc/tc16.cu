@@ -8,9 +8,8 @@
 // lo = fp16(x - hi), each with an 11-bit significand, and
 // D = A_hi B_hi + A_hi B_lo + A_lo B_hi keeps ~22 bits of the product (the
 // same as 3 x TF32, at twice the tensor rate and half the shared memory).
-// FP16's range is narrow: every row of A is scaled by a power of two so its
-// largest component lies in [0.5, 1) before the split. Matrix entries are at
-// most 1 in magnitude and need no scaling. In the epilogue the large and the
+// FP16's range is narrow: every row of A and the matrix are scaled by powers of
+// two before the split (kOperandBits). In the epilogue the large and the
 // small products (kept in separate TMEM columns, because the accumulation
 // rounds toward zero) are summed in registers and each group is rescaled to
 // its input norm -- a fused block is unitary -- which also undoes the row
@@ -140,8 +139,7 @@ __global__ void __launch_bounds__(kTcThreads * tc16_rows<K>(), Tc16Occ<K>::value
   gather(tile);
 
   for (; tile < p.n_tiles; tile += gridDim.x) {
-    // row scale: largest component into [0.5, 1); max and norm in four
-    // independent chains
+    // row scale; max and norm in four independent chains
     float m4[4] = {0.f, 0.f, 0.f, 0.f}, s4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int u = 0; u < DH; u++) {
@@ -161,9 +159,7 @@ __global__ void __launch_bounds__(kTcThreads * tc16_rows<K>(), Tc16Occ<K>::value
         nin += red_in[2 * pt + 1];
       }
     }
-    int e = 0;
-    if (mx > 0.f) frexpf(mx, &e);
-    const float sc = ldexpf(1.f, -e);
+    const float sc = row_scale(mx);
     // hi/lo rows: amplitudes 4c..4c+3 fill the 16-byte row of core matrix c
 #pragma unroll
     for (int cl = 0; cl < DH / 4; cl++) {
@@ -234,7 +230,7 @@ __global__ void __launch_bounds__(kTcThreads * tc16_rows<K>(), Tc16Occ<K>::value
       for (int o = 1; o < TPR; o++) nout += red_out[(tid + o * kTcThreads) % NT];
     }
     // unitary block: the group keeps its input norm (this also undoes the row scale)
-    const float f = nout > 0.f ? sqrtf(nin / nout) : 1.f;
+    const float f = norm_ratio(nin, nout);
     // pass 2: scale and store, 8 amplitudes per chunk
 #pragma unroll
     for (int hh = 0; hh < 2 * DH / 16; hh++) {
@@ -313,7 +309,7 @@ cudaError_t run_tc16(float2 *a, int n, const Block &b, const void *dev_b, int *e
 
 size_t tc16_b_bytes(int k) { return 2u * (size_t)(2 << k) * (size_t)(2 << k) * 2u; }
 
-// B = real embedding of U, split into FP16 hi/lo, in the 16-bit core-matrix
+// B = real embedding of U, scaled (kOperandBits) and split into FP16 hi/lo, in the 16-bit core-matrix
 // layout (row r, column c at (r/8) * (KR/8) * 64 + (c/8) * 64 + (r%8) * 8 + c%8 halves).
 void tc16_build_b(const Block &b, void *out) {
   const int D = 1 << b.k, KR = 2 * D;
@@ -348,7 +344,7 @@ void tc16_build_b(const Block &b, void *out) {
       const float vals[2][2] = {{(float)u.real(), (float)-u.imag()}, {(float)u.imag(), (float)u.real()}};
       for (int i = 0; i < 2; i++)
         for (int j = 0; j < 2; j++) {
-          const float x = vals[i][j];
+          const float x = vals[i][j] * (float)(1 << kOperandBits);
           const __half hi = __float2half_rn(x);
           const __half lo = __float2half_rn(x - __half2float(hi));
           h[at(2 * r + i, 2 * s + j)] = hi;

@@ -289,9 +289,7 @@ __global__ void __launch_bounds__(kTcThreads, tc16x_occ<K>())
     }
     const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
     const float nin = (s4[0] + s4[1]) + (s4[2] + s4[3]);
-    int e = 0;
-    if (mx > 0.f) frexpf(mx, &e);
-    const float sc = ldexpf(1.f, -e);
+    const float sc = row_scale(mx);
     // slots 4c..4c+3 (registers 2c, 2c + 1) fill the 16-byte row of core matrix c
 #pragma unroll
     for (int c = 0; c < D / 4; c++) {
@@ -349,7 +347,7 @@ __global__ void __launch_bounds__(kTcThreads, tc16x_occ<K>())
       }
     }
     const float nout = (o4[0] + o4[1]) + (o4[2] + o4[3]);
-    const float f = nout > 0.f ? sqrtf(nin / nout) : 1.f;
+    const float f = norm_ratio(nin, nout);
     // 8 slots (4 registers) at a time: scale, exchange back, store
 #pragma unroll
     for (int hh = 0; hh < KR / 16; hh++) {
@@ -605,9 +603,7 @@ __global__ void __launch_bounds__(x6::kThreads, 1)
       mx = fmaxf(mx, red_in[u][2 * (tid ^ kTcThreads)]);
       nin += red_in[u][2 * (tid ^ kTcThreads) + 1];
       if (h == 0) nin_row[u][r] = nin;
-      int e = 0;
-      if (mx > 0.f) frexpf(mx, &e);
-      const float sc = ldexpf(1.f, -e);
+      const float sc = row_scale(mx);
       // slot 2 q + c (register q, element c) holds K = 64 h + 4 q + 2 c (re)
       // and + 1 (im): column 32 h + 2 q + c of its half
       uint32_t hi[32], lo[32];
@@ -659,7 +655,7 @@ __global__ void __launch_bounds__(x6::kThreads, 1)
       x6::pair_sync(warp & 3);
       nout += red_out[u][tid ^ kTcThreads];
       const float nin = nin_row[u][r];
-      const float f = nout > 0.f ? sqrtf(nin / nout) : 1.f;
+      const float f = norm_ratio(nin, nout);
       const uint64_t cur_base = tile_base(tile);
       // 8 slots (4 registers) at a time: scale, exchange back, store
 #pragma unroll
