@@ -298,6 +298,7 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
     return fail(QS_EUNSUPPORTED, "qs_apply_circuit: global bits (opts.n_global) need a sharded runner; "
                                  "qs_plan plans their exchanges");
   DeviceGuard dg(st->device);
+  const bool by_rules = (flags & QS_PGO_RULES) && !(flags & QS_PGO_MEASURED);
   // fold the timings of an earlier profiled call that has finished
   fold_records(st, false);
   if (flags & QS_PGO_MEASURED) {
@@ -311,29 +312,59 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
     flags = rules_select(st->n, st->dtype == QS_C128, gates, n_gates, o, flags);
   }
 
+  const bool c128 = st->dtype == QS_C128;
+  const int ab = amp_bytes(st);
+  const bool prof = flags & QS_PROFILE;
+  // tensor-core tile passes where the rules choose the kernels (explicit flags
+  // run the blocks they ask for): not where each block is timed (their times
+  // are what the other activators learn from), nor where the options ask for
+  // a kernel
+  bool tiles = by_rules && !c128 && !prof && st->n > kTcTileBits && (flags & QS_TC) && o.threads == 0 &&
+               o.tc_exchange == 0 && o.tc_precision == 0;
   std::vector<Block> plan;
   PlanStats stats;
   std::string err;
   int8_t perm[QS_MAX_QUBITS];
-  std::memcpy(perm, st->perm, sizeof(perm));
-  s = build_plan(st->n, gates, n_gates, flags, o, perm, plan, stats, err, st->dtype == QS_C128);
-  if (s != QS_OK) return fail(s, "qs_apply_circuit: " + err);
+  for (;;) {
+    std::memcpy(perm, st->perm, sizeof(perm));
+    s = build_plan(st->n, gates, n_gates, flags, o, perm, plan, stats, err, c128, true, false, tiles);
+    if (s != QS_OK) return fail(s, "qs_apply_circuit: " + err);
+    if (!tiles) break;
+    // their operands take more device memory than single blocks': without it
+    // the call runs block by block
+    size_t need = operand_program_bytes(plan);
+    for (const Block &b : plan) need += dev_operand_bytes(b) + ((block_dev_matrix_bytes(b, c128) + 255) & ~(size_t)255);
+    unsigned char *dm = (unsigned char *)st->d_mats;
+    if (grow(dm, st->mats_cap, need) == cudaSuccess) {
+      st->d_mats = dm;
+      break;
+    }
+    st->d_mats = nullptr;
+    cudaGetLastError();
+    tiles = false;
+  }
   record_counters(st, gates, n_gates);
 
-  const bool c128 = st->dtype == QS_C128;
-  const int ab = amp_bytes(st);
-  const bool prof = flags & QS_PROFILE;
   // narrow states: every block in one launch (not for plain per-gate runs,
   // nor where each block is timed)
   const bool resident = !c128 && !prof && (flags & (QS_FUSE | QS_DIAG)) && o.threads == 0 && o.tc_max_ctas == 0 &&
                         resident_applies(plan, st->n);
   // matrices of wide dense blocks: one pinned staging buffer, one copy
-  size_t mat_bytes = 0;
+  size_t mat_bytes = 0, operand_bytes = 0;
   std::vector<size_t> mat_off(plan.size(), (size_t)-1);
   for (size_t i = 0; i < plan.size(); i++)
     if (!resident && block_needs_dev_matrix(plan[i], c128)) {
       mat_off[i] = mat_bytes;
       mat_bytes += (block_dev_matrix_bytes(plan[i], c128) + 255) & ~(size_t)255;
+    }
+  // tensor-core tile passes: their gates in the same upload, the operands made
+  // from them behind it
+  const size_t prog_off = mat_bytes;
+  if (tiles) mat_bytes += (operand_program_bytes(plan) + 255) & ~(size_t)255;
+  for (size_t i = 0; i < plan.size(); i++)
+    if (const size_t ob = dev_operand_bytes(plan[i])) {
+      mat_off[i] = mat_bytes + operand_bytes;
+      operand_bytes += ob;
     }
   bool any_tc = false;
   for (const Block &b : plan) any_tc |= b.tc;
@@ -356,22 +387,27 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
     }
     size_t cap_bytes = st->mats_cap;
     unsigned char *dm = (unsigned char *)st->d_mats;
-    if (mat_bytes > cap_bytes) {
+    if (mat_bytes + operand_bytes > cap_bytes) {
       dev_free(dm);
       dm = nullptr;
       st->d_mats = nullptr;
       st->mats_cap = 0;
-      e = dev_malloc((void **)&dm, mat_bytes);
+      e = dev_malloc((void **)&dm, mat_bytes + operand_bytes);
       if (e != cudaSuccess) return fail(QS_ENOMEM, "matrix buffer allocation failed");
       st->d_mats = dm;
-      st->mats_cap = mat_bytes;
+      st->mats_cap = mat_bytes + operand_bytes;
     }
     parallel_blocks(plan.size(), 1e-3 * (double)mat_bytes, [&](size_t i) {
-      if (mat_off[i] != (size_t)-1) fill_dev_matrix(plan[i], c128, (unsigned char *)st->h_mats + mat_off[i]);
+      if (mat_off[i] != (size_t)-1 && !dev_operand_bytes(plan[i]))
+        fill_dev_matrix(plan[i], c128, (unsigned char *)st->h_mats + mat_off[i]);
     });
+    if (operand_bytes) fill_operand_program(plan, (unsigned char *)st->h_mats + prog_off);
     e = cudaMemcpyAsync(st->d_mats, st->h_mats, mat_bytes, cudaMemcpyHostToDevice, st->stream);
     if (e != cudaSuccess) return cuda_fail(st, e, "qs_apply_circuit");
     e = cudaEventRecord(st->mats_copied, st->stream);
+    if (e == cudaSuccess && operand_bytes)
+      e = build_dev_operands((unsigned char *)st->d_mats + prog_off, (unsigned char *)st->d_mats + mat_bytes, operand_bytes,
+                             st->stream);
     if (e != cudaSuccess) return cuda_fail(st, e, "qs_apply_circuit");
   }
 

@@ -353,7 +353,8 @@ const DevInfo &dev_info() {
 }
 
 bool block_needs_dev_matrix(const Block &b, bool c128) {
-  if (b.kind == BK_TILE || b.kind == BK_PHASE) return true;
+  if (b.kind == BK_TILE) return !b.tc;
+  if (b.kind == BK_PHASE) return true;
   if (b.kind != BK_DENSE) return false;
   return b.tc || b.k == 6 || (c128 && b.k == 5);
 }
@@ -396,6 +397,7 @@ void fill_dev_matrix(const Block &b, bool c128, void *host_out) {
 cudaError_t launch_block_with_matrix(void *amps, int n, bool c128, const Block &b, const void *dev_mat,
                                      int *err, cudaStream_t s, int threads, LaunchShape *shape) {
   if (threads <= 0) threads = 256;
+  if (b.kind == BK_TILE && b.tc) return run_tc_tile((float2 *)amps, n, b, dev_mat, err, s, shape);
   if (b.kind == BK_TILE) return run_tile(amps, n, c128, b, dev_mat, s);
   if (b.kind == BK_PHASE) return run_phase(amps, n, c128, b, dev_mat, s, shape);
   if (b.kind == BK_DENSE && b.tc && c128)
@@ -406,6 +408,8 @@ cudaError_t launch_block_with_matrix(void *amps, int n, bool c128, const Block &
   if (c128) return run_block<double2>((double2 *)amps, n, b, dev_mat, s, threads);
   return run_block<float2>((float2 *)amps, n, b, dev_mat, s, threads);
 }
+
+size_t dev_operand_bytes(const Block &b) { return b.kind == BK_TILE && b.tc ? tc_tile_mats(b) * kTcTileBBytes : 0; }
 
 cudaError_t launch_block(void *amps, int n, bool c128, const Block &b, cudaStream_t s, int threads) {
   return launch_block_with_matrix(amps, n, c128, b, nullptr, nullptr, s, threads);
@@ -594,6 +598,7 @@ __global__ void __launch_bounds__(256) k_distance(const Ta *__restrict__ a, cons
 }
 
 template <typename T> size_t param_bytes_t(const Block &b) {
+  if (b.kind == BK_TILE && b.tc) return operand_program_bytes({b});
   if (b.kind == BK_TILE) return 2 * sizeof(T *) + sizeof(long long) + tile_desc_bytes(b, sizeof(T) == 16);
   if (b.kind == BK_PHASE) return 2 * sizeof(T *) + sizeof(long long) + phase_desc_bytes(b, sizeof(T) == 16);
   if (b.kind == BK_PERMUTE) return sizeof(T *) + sizeof(long long) + 2 * sizeof(int);

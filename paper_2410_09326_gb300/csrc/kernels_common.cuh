@@ -213,6 +213,13 @@ void tc16_build_b(const Block &b, void *out);
 cudaError_t run_dense_tc16(float2 *a, int n, const Block &b, const void *dev_b, int *err, cudaStream_t s,
                            LaunchShape *shape);
 
+// Tile passes on the tensor cores (tc_tile.cu): a BK_TILE block with tc has
+// tc_tile_mats products in all, each a B operand of kTcTileBBytes.
+constexpr size_t kTcTileBBytes = 2 * 64 * 64 * 2;
+size_t tc_tile_mats(const Block &b);
+cudaError_t run_tc_tile(float2 *a, int n, const Block &b, const void *dev_b, int *err, cudaStream_t s,
+                        LaunchShape *shape);
+
 // complex128 blocks on the tensor cores (tc64.cu), k = 4, 5: dev_b holds
 // tc64_b_bytes(k) bytes written by tc64_build_b.
 size_t tc64_b_bytes(int k);

@@ -180,19 +180,21 @@ void greedy_groups(const std::vector<qs_gate> &pg, const std::vector<int> &idx, 
 // followed by `horizon` gates of plain first-fit placement, and the choice
 // whose roll-out ends with the fewest blocks -- then the narrowest recent
 // blocks -- is kept; ties keep the earliest candidate (first fit). Placement
-// obeys the same commutation rule and width limits as greedy_groups.
-// limit(all_diag_block_and_gate) is the width bound. With free_joins a gate
-// whose first candidate needs no further qubit for it joins that one without
-// roll-outs: it widens nothing and holds later gates back the least.
-template <typename Limit>
+// obeys the same commutation rule as greedy_groups, and the limits that
+// fits(group, gate) states. With free_joins a gate whose first candidate needs
+// no further qubit for it joins that one without roll-outs: it widens nothing
+// and holds later gates back the least.
+struct LookGroup {
+  uint64_t qmask, tmask;  // its qubits; those some member acts on non-diagonally
+  bool all_diag;
+};
+
+template <typename Fits>
 void lookahead_groups(const std::vector<qs_gate> &pg, const std::vector<int> &idx, std::vector<Pending> &groups,
-                      Limit limit, int horizon, int tail_blocks, bool free_joins) {
-  struct LG {
-    uint64_t qmask;
-    bool all_diag;
-  };
+                      Fits fits_gate, int horizon, int tail_blocks, bool free_joins) {
+  using LG = LookGroup;
   struct GI {
-    uint64_t gmask;
+    uint64_t gmask, gt;
     bool gdiag;
     int nq;
     int q[6];
@@ -203,13 +205,14 @@ void lookahead_groups(const std::vector<qs_gate> &pg, const std::vector<int> &id
   for (int i = 0; i < N; i++) {
     const qs_gate &g = pg[idx[i]];
     GI &x = info[i];
-    x.gmask = 0;
+    x.gmask = x.gt = 0;
     x.gdiag = op_info(g.op).diagonal;
     x.nq = g.nq;
     for (int j = 0; j < g.nq; j++) {
       x.q[j] = g.q[j];
       x.dq[j] = gate_diag_on(g, j);
       x.gmask |= 1ull << g.q[j];
+      if (!x.dq[j]) x.gt |= 1ull << g.q[j];
     }
   }
   auto lower_of = [](const GI &x, const int *la, const int *ln) {
@@ -217,12 +220,11 @@ void lookahead_groups(const std::vector<qs_gate> &pg, const std::vector<int> &id
     for (int j = 0; j < x.nq; j++) lower = std::max(lower, x.dq[j] ? ln[x.q[j]] : la[x.q[j]]);
     return lower;
   };
-  auto fits = [&](const LG &b, const GI &x) {
-    return popcount64(b.qmask | x.gmask) <= limit(b.all_diag && x.gdiag);
-  };
+  auto fits = [&](const LG &b, const GI &x) { return fits_gate(b, LG{x.gmask, x.gt, x.gdiag}); };
   auto place = [](std::vector<LG> &G, int *la, int *ln, const GI &x, int ch) {
-    if (ch == (int)G.size()) G.push_back({0, true});
+    if (ch == (int)G.size()) G.push_back({0, 0, true});
     G[ch].qmask |= x.gmask;
+    G[ch].tmask |= x.gt;
     G[ch].all_diag = G[ch].all_diag && x.gdiag;
     for (int j = 0; j < x.nq; j++) {
       la[x.q[j]] = std::max(la[x.q[j]], ch);
@@ -272,6 +274,7 @@ void lookahead_groups(const std::vector<qs_gate> &pg, const std::vector<int> &id
     Pending &p = groups[ch];
     p.members.push_back(idx[i]);
     p.qmask |= x.gmask;
+    p.tmask |= x.gt;
     p.all_diag = p.all_diag && x.gdiag;
   }
 }
@@ -650,14 +653,164 @@ qs_status tile_plan(int n, const std::vector<qs_gate> &pg, const std::vector<int
   return QS_OK;
 }
 
+// Cost of a tile pass of b blocks, in launches of a single block of up to five
+// targets. Measured 0.45 + 0.4 b: at 27 qubits, where a block is an HBM pass,
+// 80 for the 30-qubit random circuit's 45 passes with 151 blocks (125 blocks
+// one by one), and as much at 19 qubits, where launches and latency count.
+double tc_tile_cost(size_t b) { return 0.45 + 0.4 * (double)b; }
+
+// Tensor-core tile passes (tc_tile.cu): gates grouped as in tile_plan into
+// passes whose non-diagonal qubits fit a tile of kTcTileBits, each pass's gates into
+// blocks of at most five qubits inside the tile and kTcTileSel outside it
+// (there they act diagonally: the bits pick the matrix).
+struct TcPass {
+  uint64_t tile = 0;
+  bool single = false;  // its blocks run one by one
+  std::vector<Pending> blocks;
+};
+
+// A pass whose gates cost less as blocks of K qubits one by one stays that.
+// Returns the pass's cost. search: blocks by first fit or by roll-outs,
+// whichever are fewer.
+double tc_tile_blocks(int n, const std::vector<qs_gate> &pg, const Pending &pass, int K, bool search, TcPass &out) {
+  uint64_t t = pass.tmask | ((1ull << kTileLowBits) - 1);
+  for (int q = 0; q < n && popcount64(t) < kTcTileBits; q++) t |= 1ull << q;
+  out.tile = t;
+  auto fits = [&](uint64_t q) { return popcount64(q & t) <= 5 && popcount64(q & ~t) <= kTcTileSel; };
+  greedy_groups(pg, pass.members, out.blocks,
+                [&](const Pending &p, int, uint64_t gmask, uint64_t, bool) { return fits(p.qmask | gmask); });
+  if (search) {
+    std::vector<Pending> alt;
+    lookahead_groups(
+        pg, pass.members, alt, [&](const LookGroup &a, const LookGroup &b) { return fits(a.qmask | b.qmask); }, 40, 3,
+        true);
+    if (alt.size() < out.blocks.size()) out.blocks.swap(alt);
+  }
+  std::vector<Pending> single;
+  greedy_groups(pg, pass.members, single, [&](const Pending &p, int, uint64_t gmask, uint64_t, bool) {
+    return popcount64(p.qmask | gmask) <= K;
+  });
+  if ((double)single.size() <= tc_tile_cost(out.blocks.size())) {
+    out.single = true;
+    out.blocks.swap(single);
+    return (double)out.blocks.size();
+  }
+  return tc_tile_cost(out.blocks.size());
+}
+
+// The cheapest of a few groupings into passes; returns its cost. The roll-outs
+// over blocks save one in seven at 0.4 us of host time a gate, those over
+// passes one pass and one block in ten more at 3 us: on layered circuits a
+// launch of a single block takes 30, 60, 120 and 250 us at 23 to 26 qubits, so
+// that the first pay from 23 qubits on and the second from 26.
+constexpr int kPassSearchBits = 26;
+
+double tc_tile_passes(int n, const std::vector<qs_gate> &pg, const std::vector<int> &all, int K, bool search,
+                      std::vector<TcPass> &out) {
+  const uint64_t low = (1ull << kTileLowBits) - 1;
+  auto first_fit = [&](std::vector<Pending> &passes) {
+    greedy_groups(pg, all, passes, [&](const Pending &p, int, uint64_t, uint64_t gt, bool) {
+      return popcount64(p.tmask | low | gt) <= kTcTileBits;
+    });
+  };
+  if (!search || n < kPassSearchBits) {
+    std::vector<Pending> passes;
+    first_fit(passes);
+    out.resize(passes.size());
+    std::vector<double> cost(passes.size());
+    parallel_for(passes.size(), search ? 0.4 * (double)all.size() : 0.0,
+                 [&](size_t i) { cost[i] = tc_tile_blocks(n, pg, passes[i], K, search, out[i]); });
+    double total = 0;
+    for (double c : cost) total += c;
+    return total;
+  }
+  struct Variant {
+    int horizon, tail;
+  };
+  const Variant variants[] = {{0, 0}, {60, 1}, {60, 2}, {40, 2}};
+  std::vector<TcPass> alt[4];
+  double total[4] = {0, 0, 0, 0};
+  run_tasks(4, [&](size_t v) {
+    std::vector<Pending> passes;
+    if (v == 0) {
+      first_fit(passes);
+    } else {
+      lookahead_groups(
+          pg, all, passes,
+          [&](const LookGroup &a, const LookGroup &b) { return popcount64(a.tmask | low | b.tmask) <= kTcTileBits; },
+          variants[v].horizon, variants[v].tail, false);
+    }
+    alt[v].resize(passes.size());
+    for (size_t i = 0; i < passes.size(); i++) total[v] += tc_tile_blocks(n, pg, passes[i], K, true, alt[v][i]);
+  });
+  size_t best = 0;
+  for (size_t v = 1; v < 4; v++)
+    if (total[v] < total[best]) best = v;
+  out.swap(alt[best]);
+  return total[best];
+}
+
+// A member of a tensor-core tile pass; false when all its gates are the
+// identity.
+bool finish_tile_member(const std::vector<qs_gate> &pg, const Pending &p, uint64_t tile, Block &out) {
+  out = Block();
+  out.kind = BK_DENSE;
+  out.k = 5;
+  out.n_gates = (int)p.members.size();
+  uint64_t t = p.qmask & tile;
+  for (int q = 0; popcount64(t) < 5; q++)  // widened by an identity, bit 0 first (16-byte accesses)
+    if ((tile >> q) & 1) t |= 1ull << q;
+  int w = 0;
+  for (int q = 0; q < 64; q++) {
+    if ((t >> q) & 1) out.q[w++] = q;
+    if ((p.qmask & ~tile) >> q & 1) out.sel[out.nsel++] = q;
+  }
+  const int variants = 1 << out.nsel;
+  out.skip = (1u << variants) - 1;
+  out.gates.reserve(p.members.size());
+  std::vector<cd> G;
+  for (int gi : p.members) {
+    const qs_gate &g = pg[gi];
+    gate_full_matrix(g, G);
+    const int d = 1 << g.nq;
+    Block::Member m = {(int8_t)g.nq, {0, 0, 0}};
+    for (int j = 0; j < g.nq; j++) {
+      const int at = pos_of(out.q, 5, g.q[j]);
+      m.at[j] = (int8_t)(at >= 0 ? at : -1 - pos_of(out.sel, out.nsel, g.q[j]));
+    }
+    // the variants in which the gate does something: rows and columns with
+    // the outer bits at the variant's values
+    for (int v = 0; v < variants; v++) {
+      if (!((out.skip >> v) & 1)) continue;
+      bool identity = true;
+      for (int r = 0; r < d && identity; r++) {
+        bool in = true;
+        for (int j = 0; j < g.nq; j++)
+          if (m.at[j] < 0 && ((r >> j) & 1) != ((v >> (-1 - m.at[j])) & 1)) in = false;
+        for (int c = 0; c < d && in && identity; c++) {
+          const cd z = G[(size_t)r * d + c];
+          identity = r == c ? is_one(z) : is_zero(z);
+        }
+      }
+      if (!identity) out.skip &= ~(1u << v);
+    }
+    out.mat.insert(out.mat.end(), G.begin(), G.end());
+    out.gates.push_back(m);
+  }
+  return out.skip != (1u << variants) - 1;
+}
+
 // Fusion and classification of the physical gates pg[idx...] (one segment
 // of the circuit between global-tier exchanges); appends the blocks.
 qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<int> &all, uint64_t flags,
-                       const qs_opts &opts, int D, int K, bool c128, bool allow_phase, bool repeated,
+                       const qs_opts &opts, int D, int K, bool c128, bool allow_phase, bool repeated, bool tc_tiles,
                        std::vector<Block> &plan, std::string &err) {
   const bool fuse = flags & QS_FUSE;
   const bool dfuse = flags & QS_DIAG;
   std::vector<Pending> groups;
+  std::vector<TcPass> passes;
+  bool tiled_tc = false;
+  double tiled_cost = 0;
   const bool tiled = (flags & QS_TILE) && n > tile_bits_of(opts, c128);
   if (tiled) {
     std::vector<Block> tplan;
@@ -680,6 +833,9 @@ qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<
     const bool phase_ok = dfuse && allow_phase && n > QS_MAX_DIAG;
     const int dlimit = phase_ok ? 64 : D;
     auto limit = [&](bool nd) { return nd ? (dfuse ? dlimit : std::max(K, 1)) : K; };
+    auto fits = [&](const LookGroup &a, const LookGroup &b) {
+      return popcount64(a.qmask | b.qmask) <= limit(a.all_diag && b.all_diag);
+    };
     auto first_fit = [&](std::vector<Pending> &g) {
       greedy_groups(pg, all, g, [&](const Pending &p, int, uint64_t gmask, uint64_t, bool gdiag) {
         return popcount64(p.qmask | gmask) <= limit(p.all_diag && gdiag);
@@ -694,7 +850,15 @@ qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<
     // gate and sometimes save a few blocks more at 6 targets (98 instead of
     // 107 for the 30-qubit random circuit): from 27 qubits on (25).
     const int wide = n + (c128 ? 1 : 0);
-    if (opts.fuse_lookahead > 0 && (wide >= kSearchBits || repeated)) {
+    const bool search = opts.fuse_lookahead > 0 && (wide >= kSearchBits || repeated);
+    if (tc_tiles) {
+      tiled_cost = tc_tile_passes(n, pg, all, K, search, passes);
+      first_fit(groups);
+      // not searched where no search (it saves one block in six) would change the choice
+      tiled_tc = tiled_cost < (search ? 0.8 : 1.0) * (double)groups.size();
+      if (!tiled_tc && search) groups.clear();
+    }
+    if (search && !tiled_tc) {
       // no horizon or tie-break (by the width of the last 6 or 12 blocks) is
       // best on every circuit: first fit and several roll-outs run side by
       // side on host threads, and the grouping with the fewest blocks is
@@ -711,7 +875,7 @@ qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<
       std::vector<std::vector<Pending>> alt(count);
       auto one = [&](size_t v) {
         if (v == 0) first_fit(alt[0]);
-        else lookahead_groups(pg, all, alt[v], limit, variants[v].horizon, variants[v].tail, variants[v].free_joins);
+        else lookahead_groups(pg, all, alt[v], fits, variants[v].horizon, variants[v].tail, variants[v].free_joins);
       };
       if (repeated) {  // many circuits are planned one after the other: threads would cost more than they save
         for (size_t v = 0; v < count; v++) one(v);
@@ -722,9 +886,60 @@ qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<
       for (size_t v = 1; v < count; v++)
         if (alt[v].size() < alt[best].size()) best = v;
       groups.swap(alt[best]);
-    } else {
+      tiled_tc = tc_tiles && tiled_cost < (double)groups.size();
+    } else if (!tc_tiles) {
       first_fit(groups);
     }
+  }
+
+  // (2b) tensor-core tile passes instead, where they cost less
+  if (tiled_tc) {
+    std::vector<std::pair<size_t, size_t>> at;  // (pass, block)
+    double us = 0;
+    for (size_t i = 0; i < passes.size(); i++)
+      for (size_t j = 0; j < passes[i].blocks.size(); j++) {
+        const Pending &p = passes[i].blocks[j];
+        at.push_back({i, j});
+        us += (passes[i].single ? 1.3 : 0.3) * (double)p.members.size();
+      }
+    std::vector<Block> done(at.size());
+    std::vector<char> keep(at.size(), 0);
+    parallel_for(at.size(), us, [&](size_t x) {
+      const TcPass &t = passes[at[x].first];
+      const Pending &p = t.blocks[at[x].second];
+      keep[x] = t.single ? finish_block(pg, p, true, done[x], D) : finish_tile_member(pg, p, t.tile, done[x]);
+    });
+    for (size_t x = 0; x < at.size();) {
+      const size_t i = at[x].first;
+      if (passes[i].single) {
+        if (keep[x]) plan.push_back(std::move(done[x]));
+        x++;
+        continue;
+      }
+      Block b;
+      auto open = [&] {
+        b = Block();
+        b.kind = BK_TILE;
+        b.tc = true;
+        b.k = kTcTileBits;
+        b.meta = 5;
+        int w = 0;
+        for (int q = 0; q < 64; q++)
+          if ((passes[i].tile >> q) & 1) b.tile_q[w++] = q;
+      };
+      open();
+      for (; x < at.size() && at[x].first == i; x++) {
+        if (!keep[x]) continue;
+        if (b.sub.size() == (size_t)kTcTileMaxBlocks) {
+          plan.push_back(std::move(b));
+          open();
+        }
+        b.n_gates += done[x].n_gates;
+        b.sub.push_back(std::move(done[x]));
+      }
+      if (!b.sub.empty()) plan.push_back(std::move(b));
+    }
+    return QS_OK;
   }
 
   // (3) products and classification
@@ -778,7 +993,7 @@ double block_bytes(const Block &b, int n, int amp_bytes) {
 
 qs_status build_plan(int n, const qs_gate *gates, size_t n_gates, uint64_t flags,
                      const qs_opts &opts, int8_t *perm, std::vector<Block> &plan,
-                     PlanStats &stats, std::string &err, bool c128, bool allow_phase, bool repeated) {
+                     PlanStats &stats, std::string &err, bool c128, bool allow_phase, bool repeated, bool tc_tiles) {
   plan.clear();
   stats = PlanStats();
   stats.gates_in = (int)n_gates;
@@ -979,7 +1194,7 @@ qs_status build_plan(int n, const qs_gate *gates, size_t n_gates, uint64_t flags
     const size_t seg_end = sgi < cuts.size() ? cuts[sgi] : pg.size();
     std::vector<int> idx;
     for (size_t i = seg_begin; i < seg_end; i++) idx.push_back((int)i);
-    qs_status st = plan_segment(n, pg, idx, flags, opts, D, K, c128, allow_phase, repeated, plan, err);
+    qs_status st = plan_segment(n, pg, idx, flags, opts, D, K, c128, allow_phase, repeated, tc_tiles, plan, err);
     if (st != QS_OK) return st;
     if (sgi < cuts.size()) {
       Block b;
@@ -995,6 +1210,11 @@ qs_status build_plan(int n, const qs_gate *gates, size_t n_gates, uint64_t flags
   }
   const bool tf32 = opts.tc_precision == 1;
   for (Block &b : plan) {
+    if (b.kind == BK_TILE && b.tc) {
+      b.withhold_commit = opts.test_wait_timeout != 0;
+      b.tc_max_ctas = opts.tc_max_ctas;
+      continue;
+    }
     // complex128 blocks run on FP16 digit planes (tc64.cu), 4 and 5 targets
     b.tc = (flags & QS_TC) && b.kind == BK_DENSE && b.k >= 4 && b.k <= (tf32 || c128 ? 5 : 6);
     b.tc_tf32 = b.tc && tf32 && !c128;

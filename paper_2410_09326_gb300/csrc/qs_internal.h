@@ -48,6 +48,9 @@ enum BlockKind : uint8_t { BK_DENSE = 0, BK_DIAG = 1, BK_PERMUTE = 2, BK_TILE = 
 constexpr int kMaxFixed = 24;  // targets + controls handled by the index insert
 constexpr int kMaxTileBits = 14;  // widest shared-memory tile (QS_TILE)
 constexpr int kTileLowBits = 4;   // contiguous low bits every tile includes (128-byte c64 runs)
+constexpr int kTcTileBits = 12;       // tile of a tensor-core pass (tc_tile.cu): 32 KiB
+constexpr int kTcTileMaxBlocks = 32;  // its blocks in one launch
+constexpr int kTcTileSel = 2;         // bits outside the tile that pick a block's matrix
 
 struct Block {
   BlockKind kind = BK_DENSE;
@@ -70,6 +73,19 @@ struct Block {
   // dense targets inside the tile, diagonal qubits and controls anywhere
   int tile_q[kMaxTileBits] = {0};
   std::vector<Block> sub;
+  // tensor-core tile passes (BK_TILE with tc): a member has five targets and
+  // is one of 2^nsel products of its gates, picked by the state's bits sel.
+  // The device forms the products: mat holds the gates' own matrices, one
+  // after the other, gates their qubits. skip: bit v is set where every gate
+  // of variant v is the identity
+  struct Member {
+    int8_t nq;
+    int8_t at[3];  // position among the targets, or -1 - j for sel[j]
+  };
+  std::vector<Member> gates;
+  int nsel = 0;
+  int sel[kTcTileSel] = {0};
+  uint32_t skip = 0;
   // phase polynomial (BK_PHASE): the block multiplies amplitude x by
   // exp(i (ph_c + sum_j ph_a[j] x_{ph_q[j]} + sum_{j<l} ph_b[j,l] x_{ph_q[j]} x_{ph_q[l]})),
   // k = ph_q.size(), ph_b upper triangle in row order, angles in (-pi, pi]
@@ -127,11 +143,12 @@ struct PlanStats {
 // Returns QS_OK or QS_EINVAL (message in err).
 // c128 selects the amplitude size the default tile width is computed for.
 // repeated: the plan will run many times, so that fusion is searched at any
-// width.
+// width. tc_tiles: tensor-core tile passes may take the place of single blocks
+// where they are estimated to be faster.
 qs_status build_plan(int n, const qs_gate *gates, size_t n_gates, uint64_t flags,
                      const qs_opts &opts, int8_t *perm, std::vector<Block> &plan,
                      PlanStats &stats, std::string &err, bool c128 = false, bool allow_phase = true,
-                     bool repeated = false);
+                     bool repeated = false, bool tc_tiles = false);
 
 // Tile width QS_TILE uses for these options and amplitude type.
 int tile_bits_of(const qs_opts &o, bool c128);
@@ -193,6 +210,13 @@ cudaError_t launch_block(void *amps, int n, bool c128, const Block &b, cudaStrea
 bool block_needs_dev_matrix(const Block &b, bool c128);
 size_t block_dev_matrix_bytes(const Block &b, bool c128);
 void fill_dev_matrix(const Block &b, bool c128, void *host_out);
+// Tensor-core tile passes read operands that a launch makes on the device from
+// their members' gates: their size (0 for other blocks), and for all passes of
+// a plan, the gates as uploaded (program) and the launch.
+size_t dev_operand_bytes(const Block &b);
+size_t operand_program_bytes(const std::vector<Block> &plan);
+void fill_operand_program(const std::vector<Block> &plan, void *out);
+cudaError_t build_dev_operands(const void *program, void *out, size_t bytes, cudaStream_t s);
 // Bytes of gate data one block ships to the device: its kernel parameters
 // (matrix or phase table included) plus any matrix upload.
 size_t block_param_bytes(const Block &b, bool c128);

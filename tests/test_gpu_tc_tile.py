@@ -1,0 +1,151 @@
+"""Tile passes on the tensor cores (complex64, several fused blocks per launch) against the oracle."""
+
+import random
+
+import numpy as np
+import pytest
+
+import circuitgen as cg
+import oracle
+import paper_2410_09326_gb300 as qs
+
+pytestmark = pytest.mark.gpu
+
+FLAGS = qs.QS_PGO_RULES
+
+
+def _layers(n, layers, seed, kinds):
+    r = random.Random(seed)
+    gates = []
+    for _ in range(layers):
+        gates += [("u3", [q], [r.uniform(0, 6.28) for _ in range(3)]) for q in range(n)]
+        q = r.sample(range(n), n)
+        for a, b, c in zip(q[::3], q[1::3], q[2::3]):
+            k = r.choice(kinds)
+            if k in ("ccx", "cswap"):
+                gates.append((k, [a, b, c]))
+            elif k in ("cx", "cz", "swap"):
+                gates.append((k, [a, b]))
+            else:
+                gates.append((k, [a, b], [r.uniform(0, 6.28)]))
+    return gates
+
+
+def _random_state(n, seed):
+    g = np.random.default_rng(seed)
+    x = g.standard_normal(1 << n) + 1j * g.standard_normal(1 << n)
+    return x / np.linalg.norm(x)
+
+
+def _run(n, gates, init, flags=FLAGS, opts=None):
+    st = qs.qs_alloc_state(n, qs.QS_C64)
+    try:
+        qs.qs_write_state(st, init.astype(np.complex64))
+        qs.qs_apply_circuit(st, qs.gates_to_array(gates), flags, opts)
+        recs = qs.qs_profile(st)[1]
+        return qs.qs_read_state(st, n, qs.QS_C64, logical_order=True).astype(np.complex128), recs
+    finally:
+        qs.qs_free_state(st)
+
+
+# the narrowest state with tiles, several tiles, one that several CTAs loop over (ctas), many;
+# controls and phases on any bit, 3-qubit gates, blocks that are the identity on some tiles
+@pytest.mark.parametrize("n,ctas,kinds", [
+    (14, 0, ["cx", "cp", "rzz", "swap"]), (14, 1, ["cx", "ccx"]),
+    (14, 3, ["ccx", "cswap", "crx"]), (15, 3, ["cx", "cz"]), (16, 5, ["ccx", "cp", "cx"]),
+    (18, 0, ["cx", "crx", "ccx"]), (20, 0, ["cx", "cz", "cp"]),
+])
+def test_against_oracle(n, ctas, kinds):
+    gates = _layers(n, 4, 31 * n + ctas, kinds)
+    init = _random_state(n, n)
+    opts = qs.qs_default_opts()
+    opts.tc_max_ctas = ctas
+    got, recs = _run(n, gates, init, FLAGS, opts)
+    tiles = [r for r in recs if r.kind == 3]
+    assert tiles and all(r.tc and r.tiles == 1 << (n - 12) for r in tiles)
+    assert all(r.ctas == (min(ctas, r.tiles) if ctas else min(r.tiles, r.ctas)) for r in tiles)
+    want, _ = oracle.simulate(cg.to_qasm(n, gates), init=init)
+    # a block's error is below 4e-7 of the state (FP16 halves, FP32 sums); they add up at most
+    assert np.linalg.norm(got - want) <= 4e-7 * sum(max(1, r.n_gates) for r in recs) ** 0.5 * 4
+
+
+def test_every_block_controlled_from_outside_the_tile():
+    """Blocks that only act where the highest bits are 1: tiles without work are left as they are."""
+    n, top = 15, [13, 14]
+    r = random.Random(5)
+    gates = []
+    for _ in range(6):
+        gates += [("cu3", [top[q % 2], q], [r.uniform(0, 6.28) for _ in range(3)]) for q in range(11)]
+        gates += [("ccx", [top[0], q, q + 1]) for q in range(0, 10, 2)]
+    init = _random_state(n, 9)
+    got, recs = _run(n, gates, init)
+    assert any(r.kind == 3 for r in recs)
+    want, _ = oracle.simulate(cg.to_qasm(n, gates), init=init)
+    assert np.linalg.norm(got - want) <= 1e-5
+    quarter = np.arange(1 << n) >> 13 == 0
+    assert np.array_equal(got[quarter].astype(np.complex64), init[quarter].astype(np.complex64))
+
+
+def test_rows_of_any_size():
+    """Groups far smaller than the rest, zero groups, NaN in one group: each keeps to itself."""
+    n = 14
+    gates = _layers(11, 3, 3, ["cx"])  # bits 0..10: one tile pass, whole tiles along the other bits
+    init = _random_state(n, 4).reshape(8, 1 << 11)
+    init[1] *= 1e-12
+    init[2] = 0
+    init[3, 5] = np.nan
+    got, recs = _run(n, gates, init.reshape(-1))
+    got = got.reshape(8, 1 << 11)
+    assert any(r.kind == 3 for r in recs)
+    text = cg.to_qasm(11, gates)
+    for i in (0, 1, 4, 5, 6, 7):
+        size = np.linalg.norm(init[i])
+        want, _ = oracle.simulate(text, init=init[i] / size)
+        assert np.linalg.norm(got[i] / size - want) <= 1e-5, i
+    assert (got[2] == 0).all() and np.isnan(got[3]).any()
+
+
+def test_profiled_calls_scarce_memory_and_explicit_flags_run_block_by_block():
+    n = 16
+    gates = _layers(n, 5, 8, ["cx", "cz"])
+    init = _random_state(n, 2)
+    before = qs.qs_memory_in_use()
+    st = qs.qs_alloc_state(n, qs.QS_C64)
+    try:
+        qs.qs_apply_circuit(st, qs.gates_to_array(gates), FLAGS | qs.QS_PROFILE)
+        assert not any(r.kind == 3 for r in qs.qs_profile(st)[1])
+        single = qs.qs_memory_in_use() - before
+    finally:
+        qs.qs_free_state(st)
+    tiled, recs = _run(n, gates, init)
+    assert any(r.kind == 3 for r in recs)
+    qs.qs_set_memory_limit(before + single)
+    try:
+        blocks, recs = _run(n, gates, init)
+    finally:
+        qs.qs_set_memory_limit(0)
+    assert not any(r.kind == 3 for r in recs)
+    assert np.linalg.norm(tiled - blocks) <= 1e-5
+    # explicit flags run the blocks they ask for
+    _, recs = _run(n, gates, init, qs.QS_VSWAP | qs.QS_FUSE | qs.QS_FUSE_K(5) | qs.QS_DIAG | qs.QS_TC)
+    assert not any(r.kind == 3 for r in recs)
+
+
+def test_timeout_is_reported():
+    n = 14
+    gates = qs.gates_to_array(_layers(n, 3, 1, ["cx"]))
+    st = qs.qs_alloc_state(n, qs.QS_C64)
+    try:
+        opts = qs.qs_default_opts()
+        opts.test_wait_timeout = 1
+        qs.qs_apply_circuit(st, gates, FLAGS, opts)
+        with pytest.raises(qs.QsError) as e:
+            qs.qs_norm(st)
+        assert e.value.status == qs.QS_ETIMEOUT
+        opts.test_wait_timeout = 0
+        qs.qs_set_basis(st, 0)
+        qs.qs_apply_circuit(st, gates, FLAGS, opts)
+        assert any(r.kind == 3 for r in qs.qs_profile(st)[1])
+        assert abs(qs.qs_norm(st) - 1) < 1e-5
+    finally:
+        qs.qs_free_state(st)
