@@ -397,7 +397,10 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
       st->d_mats = dm;
       st->mats_cap = mat_bytes + operand_bytes;
     }
-    parallel_blocks(plan.size(), 1e-3 * (double)mat_bytes, [&](size_t i) {
+    // (a phase polynomial's table takes about 30 us, a matrix 0.25 ns a byte of its operand)
+    double fill_us = 0.25e-3 * (double)mat_bytes;
+    for (const Block &b : plan) fill_us += b.kind == BK_PHASE ? 30 : 0;
+    parallel_blocks(plan.size(), fill_us, [&](size_t i) {
       if (mat_off[i] != (size_t)-1 && !dev_operand_bytes(plan[i]))
         fill_dev_matrix(plan[i], c128, (unsigned char *)st->h_mats + mat_off[i]);
     });
@@ -405,6 +408,7 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
     e = cudaMemcpyAsync(st->d_mats, st->h_mats, mat_bytes, cudaMemcpyHostToDevice, st->stream);
     if (e != cudaSuccess) return cuda_fail(st, e, "qs_apply_circuit");
     e = cudaEventRecord(st->mats_copied, st->stream);
+    if (e == cudaSuccess && any_tc) e = make_dev_operands(plan, mat_off, c128, st->d_mats, st->stream);
     if (e == cudaSuccess && operand_bytes)
       e = build_dev_operands((unsigned char *)st->d_mats + prog_off, (unsigned char *)st->d_mats + mat_bytes, operand_bytes,
                              st->stream);

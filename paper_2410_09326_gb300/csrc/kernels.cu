@@ -377,10 +377,8 @@ void fill_dev_matrix(const Block &b, bool c128, void *host_out) {
     phase_fill_desc(b, c128, host_out);
     return;
   }
-  if (b.tc) {
-    if (c128) tc64_build_b(b, host_out);
-    else if (b.tc_tf32) tc_build_b(b, (float *)host_out);
-    else tc16_build_b(b, host_out);
+  if (b.tc_tf32) {
+    tc_build_b(b, (float *)host_out);
     return;
   }
   for (size_t k = 0; k < b.mat.size(); k++) {

@@ -207,9 +207,10 @@ void tc_build_b(const Block &b, float *out);
 cudaError_t run_dense_tc(float2 *a, int n, const Block &b, const void *dev_b, int *err, cudaStream_t s,
                          LaunchShape *shape);
 // FP16-operand variant (tc16.cu), k = 4..6: dev_b holds tc16_b_bytes(k) bytes
-// written by tc16_build_b.
+// made by make_dev_operands: B = real embedding of U, split into FP16 hi/lo, in
+// the 16-bit core-matrix layout (row r, column c at (r/8) * (KR/8) * 64 +
+// (c/8) * 64 + (r%8) * 8 + c%8 halves).
 size_t tc16_b_bytes(int k);
-void tc16_build_b(const Block &b, void *out);
 cudaError_t run_dense_tc16(float2 *a, int n, const Block &b, const void *dev_b, int *err, cudaStream_t s,
                            LaunchShape *shape);
 
@@ -221,9 +222,8 @@ cudaError_t run_tc_tile(float2 *a, int n, const Block &b, const void *dev_b, int
                         LaunchShape *shape);
 
 // complex128 blocks on the tensor cores (tc64.cu), k = 4, 5: dev_b holds
-// tc64_b_bytes(k) bytes written by tc64_build_b.
+// tc64_b_bytes(k) bytes made by make_dev_operands: digit planes in that layout.
 size_t tc64_b_bytes(int k);
-void tc64_build_b(const Block &b, void *out);
 cudaError_t run_dense_tc64(double2 *a, int n, const Block &b, const void *dev_b, int *err, cudaStream_t s,
                            LaunchShape *shape);
 

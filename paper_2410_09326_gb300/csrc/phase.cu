@@ -207,21 +207,29 @@ template <typename T> void fill_desc_t(const Block &b, unsigned char *out) {
   PhaseHdr *h = reinterpret_cast<PhaseHdr *>(out);
   T *ltab = reinterpret_cast<T *>(out + sizeof(PhaseHdr));
   PhaseTerm<T> *terms = reinterpret_cast<PhaseTerm<T> *>(ltab + (1 << kPhaseChunkBits));
-  // table of the terms among chunk bits (constant included), in FP64
+  // table of the terms among chunk bits (constant included), in FP64. The
+  // angles double up: with bit q set, those of the bits below plus the bit's
+  // own terms, which double up the same way
   const int k = b.k;
-  for (int o = 0; o < (1 << kPhaseChunkBits); o++) {
-    double ang = b.ph_c;
-    for (int j = 0; j < k; j++) {
-      const int qj = b.ph_q[j];
-      if (qj >= kPhaseChunkBits || !((o >> qj) & 1)) continue;
-      ang += b.ph_a[j];
-      for (int l = j + 1; l < k; l++) {
-        const int ql = b.ph_q[l];
-        if (ql < kPhaseChunkBits && ((o >> ql) & 1)) ang += b.ph_b[tri_index(j, l, k)];
+  std::vector<double> ang(1 << kPhaseChunkBits), own(1 << kPhaseChunkBits);
+  ang[0] = b.ph_c;
+  for (int j = 0, q = 0; q < kPhaseChunkBits; q++) {  // j: terms of the lower bits
+    const bool has = j < k && b.ph_q[j] == q;
+    own[0] = has ? b.ph_a[j] : 0.0;
+    for (int l = 0, p = 0; p < q; p++) {
+      double pair = 0.0;
+      if (l < k && b.ph_q[l] == p) {
+        if (has) pair = b.ph_b[tri_index(l, j, k)];
+        l++;
       }
+      for (int o = 0; o < (1 << p); o++) own[(1 << p) + o] = own[o] + pair;
     }
-    ltab[o].x = (R)std::cos(ang);
-    ltab[o].y = (R)std::sin(ang);
+    for (int o = 0; o < (1 << q); o++) ang[(1 << q) + o] = ang[o] + own[o];
+    if (has) j++;
+  }
+  for (int o = 0; o < (1 << kPhaseChunkBits); o++) {
+    ltab[o].x = (R)std::cos(ang[o]);
+    ltab[o].y = (R)std::sin(ang[o]);
   }
   // counting sort by slot
   int cnt[kPhaseSlots] = {0};

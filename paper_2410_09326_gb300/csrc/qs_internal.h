@@ -210,6 +210,10 @@ cudaError_t launch_block(void *amps, int n, bool c128, const Block &b, cudaStrea
 bool block_needs_dev_matrix(const Block &b, bool c128);
 size_t block_dev_matrix_bytes(const Block &b, bool c128);
 void fill_dev_matrix(const Block &b, bool c128, void *host_out);
+// Single tensor-core blocks: makes their operands on the device, in place, from
+// the matrices that fill_dev_matrix wrote at off[i] (-1: none) behind base.
+cudaError_t make_dev_operands(const std::vector<Block> &plan, const std::vector<size_t> &off, bool c128, void *base,
+                              cudaStream_t s);
 // Tensor-core tile passes read operands that a launch makes on the device from
 // their members' gates: their size (0 for other blocks), and for all passes of
 // a plan, the gates as uploaded (program) and the launch.

@@ -87,6 +87,17 @@ template <int K> size_t tc16_smem_bytes() {
   return 2 * 128 * KR * 2 + 2 * KR * KR * 2;
 }
 
+// One entry of a matrix in B: the FP16 halves of its two columns in the real
+// embedding's row for the real (odd = 0) or the imaginary part, scaled.
+__device__ __forceinline__ void operand_halves(int odd, float re, float im, uint32_t &hi, uint32_t &lo) {
+  constexpr float s = (float)(1 << kOperandBits);
+  const float c0 = (odd ? im : re) * s, c1 = (odd ? re : -im) * s;
+  const __half2 h2 = __floats2half2_rn(c0, c1);
+  const float2 hf = __half22float2(h2);
+  hi = *reinterpret_cast<const uint32_t *>(&h2);
+  lo = pack_half2(c0 - hf.x, c1 - hf.y);
+}
+
 // The lane-exchange kernels (tc16x.cu) for a block the planner marked for
 // them (b.tc_xg); B must have been built in slot order (tc16_build_b does).
 cudaError_t run_dense_tc16x(float2 *a, int n, const Block &b, const void *dev_b, int *err, cudaStream_t s,

@@ -17,7 +17,7 @@
 //    |a_i| <= 128. The last digit's weight is 2^-55, at most half the spacing
 //    of FP64 numbers at the group's largest.
 //  - B: the real embedding of the block matrix, u = sum_j b_j 2^(-7-8j),
-//    j = 0..7, made on the host.
+//    j = 0..7 (operands.cu).
 //  - Level s = i + j = 0..7: acc_s = sum over i + j = s and the 2^(K+1) columns
 //    of a_i b_j, an integer of at most 8 * 64 * 2^14 = 2^23, so FP32 sums it
 //    exactly in any order. The terms left out (i + j >= 8) are below 2^-64 each.
@@ -339,34 +339,6 @@ cudaError_t run_tc64(double2 *a, int n, const Block &b, const void *dev_b, int *
 }  // namespace
 
 size_t tc64_b_bytes(int k) { return (size_t)kLevels * (2u << k) * (2u << k) * 2u; }
-
-// The digit planes of B, stacked along its rows -- those of the outputs with
-// the highest target 0 first, then the others -- in the 16-bit core-matrix
-// layout (row r, column c at (r/8) * (KR/8) * 64 + (c/8) * 64 + (r%8) * 8 + c%8
-// halves).
-void tc64_build_b(const Block &b, void *out) {
-  const int D = 1 << b.k, KR = 2 * D;
-  __half *hp = (__half *)out;
-  auto at = [&](int row, int col) {
-    return (size_t)(row >> 3) * (KR / 8) * 64 + (size_t)(col >> 3) * 64 + (row & 7) * 8 + (col & 7);
-  };
-  for (int r = 0; r < D; r++)
-    for (int c = 0; c < D; c++) {
-      const cd u = b.mat[(size_t)r * D + c];
-      double re = u.real() * 128.0, im = u.imag() * 128.0;
-      for (int j = 0; j < kLevels; j++) {
-        const double dr = std::nearbyint(re), di = std::nearbyint(im);
-        re = (re - dr) * 256.0;
-        im = (im - di) * 256.0;
-        const __half hr = __float2half_rn((float)dr), hi = __float2half_rn((float)di);
-        const int row = (r < D / 2 ? j * D + 2 * r : (kLevels + j) * D + 2 * r - D);
-        hp[at(row, 2 * c)] = hr;
-        hp[at(row + 1, 2 * c + 1)] = hr;
-        hp[at(row, 2 * c + 1)] = __float2half_rn((float)-di);
-        hp[at(row + 1, 2 * c)] = hi;
-      }
-    }
-}
 
 cudaError_t run_dense_tc64(double2 *a, int n, const Block &b, const void *dev_b, int *err, cudaStream_t s,
                            LaunchShape *shape) {

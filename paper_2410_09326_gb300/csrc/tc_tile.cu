@@ -378,8 +378,8 @@ static_assert(sizeof(TtGate) == 16, "16-byte words");
 
 // One product per CTA: the 32 x 32 matrix in FP64, gate by gate from the left
 // in shared memory, then B: its real embedding, rounded to FP32, scaled, split
-// into FP16 halves and laid out in the MMA's core matrices (tc16_build_b in
-// tc16.cu). Thread (warp w, lane c) updates column c of every fourth group of
+// into FP16 halves and laid out in the MMA's core matrices (as operands.cu
+// does). Thread (warp w, lane c) updates column c of every fourth group of
 // rows. Bound by the FP64 rate (two multiply-adds per clock and SM): zeros
 // and unchanged rows, which the gate's matrix shows to all threads alike, are
 // skipped. On the host these products took 1.3 ms of the 1.9 ms that the
@@ -459,12 +459,7 @@ __global__ void __launch_bounds__(128) k_tc_tile_product(const uint4 *__restrict
 #pragma unroll
     for (int e = 0; e < 4; e++) {
       const double2 u = m[row >> 1][cg * 4 + e];
-      const float re = (float)u.x * (float)(1 << kOperandBits), im = (float)u.y * (float)(1 << kOperandBits);
-      const float c0 = row & 1 ? im : re, c1 = row & 1 ? re : -im;
-      const __half2 h2 = __floats2half2_rn(c0, c1);
-      const float2 hf = __half22float2(h2);
-      hi[e] = *reinterpret_cast<const uint32_t *>(&h2);
-      lo[e] = pack_half2(c0 - hf.x, c1 - hf.y);
+      operand_halves(row & 1, (float)u.x, (float)u.y, hi[e], lo[e]);
     }
     uint4 *o = out + (row >> 3) * 64 + cg * 8 + (row & 7);
     o[0] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
