@@ -669,6 +669,30 @@ struct TcPass {
   std::vector<Pending> blocks;
 };
 
+// The gates with every one-qubit gate moved back to just before the next gate
+// on its qubit that has others, with which it then shares a block: first fit
+// would take a layer's one-qubit gates in the order they come. 82 -> 77 blocks
+// for a 19-qubit 30-layer random circuit.
+std::vector<int> one_qubit_late(const std::vector<qs_gate> &pg, const std::vector<int> &idx) {
+  std::vector<int> out, wait[64];
+  out.reserve(idx.size());
+  auto flush = [&](int q) {
+    out.insert(out.end(), wait[q].begin(), wait[q].end());
+    wait[q].clear();
+  };
+  for (int i : idx) {
+    const qs_gate &g = pg[i];
+    if (g.nq == 1) {
+      wait[g.q[0]].push_back(i);
+      continue;
+    }
+    for (int j = 0; j < g.nq; j++) flush(g.q[j]);
+    out.push_back(i);
+  }
+  for (int q = 0; q < 64; q++) flush(q);
+  return out;
+}
+
 // A pass whose gates cost less as blocks of K qubits one by one stays that.
 // Returns the pass's cost. search: blocks by first fit or by roll-outs,
 // whichever are fewer.
@@ -677,17 +701,18 @@ double tc_tile_blocks(int n, const std::vector<qs_gate> &pg, const Pending &pass
   for (int q = 0; q < n && popcount64(t) < kTcTileBits; q++) t |= 1ull << q;
   out.tile = t;
   auto fits = [&](uint64_t q) { return popcount64(q & t) <= 5 && popcount64(q & ~t) <= kTcTileSel; };
-  greedy_groups(pg, pass.members, out.blocks,
+  const std::vector<int> idx = one_qubit_late(pg, pass.members);
+  greedy_groups(pg, idx, out.blocks,
                 [&](const Pending &p, int, uint64_t gmask, uint64_t, bool) { return fits(p.qmask | gmask); });
   if (search) {
     std::vector<Pending> alt;
     lookahead_groups(
-        pg, pass.members, alt, [&](const LookGroup &a, const LookGroup &b) { return fits(a.qmask | b.qmask); }, 40, 3,
+        pg, idx, alt, [&](const LookGroup &a, const LookGroup &b) { return fits(a.qmask | b.qmask); }, 40, 3,
         true);
     if (alt.size() < out.blocks.size()) out.blocks.swap(alt);
   }
   std::vector<Pending> single;
-  greedy_groups(pg, pass.members, single, [&](const Pending &p, int, uint64_t gmask, uint64_t, bool) {
+  greedy_groups(pg, idx, single, [&](const Pending &p, int, uint64_t gmask, uint64_t, bool) {
     return popcount64(p.qmask | gmask) <= K;
   });
   if ((double)single.size() <= tc_tile_cost(out.blocks.size())) {
