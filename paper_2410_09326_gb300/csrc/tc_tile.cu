@@ -376,79 +376,134 @@ struct TtGate {
 };
 static_assert(sizeof(TtGate) == 16, "16-byte words");
 
+// Applies a gate on NT of the product's five bits: thread (warp w, lane c)
+// updates column c of every fourth group of rows. z is the gate's matrix,
+// off[l] the row bits of its index l. Zeros and unchanged rows, the same for
+// all threads, are skipped; the tests are on bits, since comparisons would
+// share the FP64 pipe.
+template <int NT>
+__device__ __forceinline__ void left_apply(double2 (&m)[32][32], const double2 *z, int tm, const int (&off)[8]) {
+  constexpr int D = 1 << NT;
+  const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
+  auto bits_zero = [](double v) { return (__double2hiint(v) << 1 | __double2loint(v)) == 0; };
+  auto is_one = [&](double2 v) {
+    return __double2hiint(v.x) == 0x3ff00000 && __double2loint(v.x) == 0 && bits_zero(v.y);
+  };
+  for (int q = w; q < (32 >> NT); q += 4) {
+    int row = q;  // the q-th row whose target bits are 0
+#pragma unroll
+    for (int j = 0; j < 5; j++)
+      if ((tm >> j) & 1) row = ((row >> j) << (j + 1)) | (row & ((1 << j) - 1));
+    double2 x[D];
+#pragma unroll
+    for (int l = 0; l < D; l++) x[l] = m[row | off[l]][c];
+#pragma unroll
+    for (int r = 0; r < D; r++) {
+      double2 s = make_double2(0.0, 0.0);
+      bool same = true, first = true;
+#pragma unroll
+      for (int l = 0; l < D; l++) {
+        const double2 g = z[r * D + l];
+        const bool re = !bits_zero(g.x), im = !bits_zero(g.y);
+        if (!re && !im) {
+          same = same && l != r;
+          continue;
+        }
+        if (is_one(g)) {
+          same = same && l == r;
+          if (first) s = x[l];
+          else s.x += x[l].x, s.y += x[l].y;
+          first = false;
+          continue;
+        }
+        same = first = false;
+        if (re) {
+          s.x = fma(g.x, x[l].x, s.x);
+          s.y = fma(g.x, x[l].y, s.y);
+        }
+        if (im) {
+          s.x = fma(-g.y, x[l].y, s.x);
+          s.y = fma(g.y, x[l].x, s.y);
+        }
+      }
+      if (!same) m[row | off[r]][c] = s;
+    }
+  }
+}
+
 // One product per CTA: the 32 x 32 matrix in FP64, gate by gate from the left
 // in shared memory, then B: its real embedding, rounded to FP32, scaled, split
 // into FP16 halves and laid out in the MMA's core matrices (as operands.cu
-// does). Thread (warp w, lane c) updates column c of every fourth group of
-// rows. Bound by the FP64 rate (two multiply-adds per clock and SM): zeros
-// and unchanged rows, which the gate's matrix shows to all threads alike, are
-// skipped. On the host these products took 1.3 ms of the 1.9 ms that the
-// 19-qubit 30-layer circuit spends there.
+// does). The next gate's matrix is fetched while one is applied. Bound by the
+// FP64 rate, two multiply-adds per clock and SM (a one-qubit gate of real and
+// imaginary entries is 4096 clocks): 65 us for the 158 products of the 19-qubit
+// 30-layer random circuit, 178 us with one loop for all gate sizes, FP64
+// comparisons and the matrix read from global memory entry by entry.
 __global__ void __launch_bounds__(128) k_tc_tile_product(const uint4 *__restrict__ prog, uint4 *__restrict__ b) {
   __shared__ double2 m[32][32];
+  __shared__ double2 z[2][64];
   const int tid = threadIdx.x, c = tid & 31, w = tid >> 5;
   const uint2 entry = reinterpret_cast<const uint2 *>(prog)[blockIdx.x];
   const uint4 *member = prog + entry.x;
   const int n_gates = (int)member->x;
-  for (int r = w; r < 32; r += 4) m[r][c] = make_double2(r == c ? 1.0 : 0.0, 0.0);
-  for (int i = 0; i < n_gates; i++) {
-    __syncthreads();
+  struct Gate {
+    int nt, tm;    // its bits inside the product
+    double2 e;     // thread i < 4^nt: entry i of its matrix
+    int off[8];
+  };
+  auto fetch = [&](int i) {
+    Gate o;
     const TtGate g = reinterpret_cast<const TtGate *>(member + 1)[i];
-    const double2 *G = reinterpret_cast<const double2 *>(member + g.mat);
-    // gate index of local row l: its target bits spread out, the outer bits fixed
-    int tm = 0, fixed = 0, nt = 0, full[8] = {0, 0, 0, 0, 0, 0, 0, 0}, off[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int j = 0; j < g.nq; j++) {
+    int fixed = 0, bit[3] = {0, 0, 0}, at[3] = {0, 0, 0};
+    o.nt = o.tm = 0;
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+      if (j >= g.nq) continue;
       if (g.at[j] < 0) {
         fixed |= (int)((entry.y >> (-1 - g.at[j])) & 1) << j;
         continue;
       }
-      tm |= 1 << g.at[j];
+      o.tm |= 1 << g.at[j];
 #pragma unroll
-      for (int l = 0; l < 8; l++)
-        if ((l >> nt) & 1) {
-          full[l] |= 1 << j;
-          off[l] |= 1 << g.at[j];
-        }
-      nt++;
+      for (int u = 0; u < 3; u++)
+        if (u == o.nt) bit[u] = 1 << j, at[u] = 1 << g.at[j];
+      o.nt++;
     }
-    const int d = 1 << nt, dg = 1 << g.nq;
-    for (int q = w; q < (32 >> nt); q += 4) {
-      int row = q;  // the q-th row whose target bits are 0
 #pragma unroll
-      for (int j = 0; j < 5; j++)
-        if ((tm >> j) & 1) row = ((row >> j) << (j + 1)) | (row & ((1 << j) - 1));
-      double2 x[8], y[8];
+    for (int l = 0; l < 8; l++) {
+      o.off[l] = 0;
 #pragma unroll
-      for (int l = 0; l < 8; l++)
-        if (l < d) x[l] = m[row | off[l]][c];
+      for (int u = 0; u < 3; u++)
+        if ((l >> u) & 1) o.off[l] |= at[u];
+    }
+    // the entry's row and column in the gate's own matrix: the outer bits fixed
+    int r = fixed, k = fixed;
 #pragma unroll
-      for (int r = 0; r < 8; r++) {
-        if (r >= d) continue;
-        double2 s = make_double2(0.0, 0.0);
-#pragma unroll
-        for (int l = 0; l < 8; l++) {
-          if (l >= d) continue;
-          const double2 z = G[(full[r] | fixed) * dg + (full[l] | fixed)];
-          if (z.x == 1.0 && z.y == 0.0) {
-            s.x += x[l].x;
-            s.y += x[l].y;
-            continue;
-          }
-          if (z.x != 0.0) {
-            s.x = fma(z.x, x[l].x, s.x);
-            s.y = fma(z.x, x[l].y, s.y);
-          }
-          if (z.y != 0.0) {
-            s.x = fma(-z.y, x[l].y, s.x);
-            s.y = fma(z.y, x[l].x, s.y);
-          }
-        }
-        y[r] = s;
+    for (int u = 0; u < 3; u++) {
+      if ((tid >> u) & 1 && u < o.nt) k |= bit[u];
+      if ((tid >> (o.nt + u)) & 1 && u < o.nt) r |= bit[u];
+    }
+    o.e = make_double2(0.0, 0.0);
+    if (tid < 1 << (2 * o.nt)) o.e = reinterpret_cast<const double2 *>(member + g.mat)[(r << g.nq) + k];
+    return o;
+  };
+  for (int r = w; r < 32; r += 4) m[r][c] = make_double2(r == c ? 1.0 : 0.0, 0.0);
+  Gate cur = fetch(0);
+  for (int i = 0; i < n_gates; i++) {
+    if (tid < 64) z[i & 1][tid] = cur.e;
+    __syncthreads();
+    Gate nxt = cur;
+    if (i + 1 < n_gates) nxt = fetch(i + 1);
+    switch (cur.nt) {
+      case 1: left_apply<1>(m, z[i & 1], cur.tm, cur.off); break;
+      case 2: left_apply<2>(m, z[i & 1], cur.tm, cur.off); break;
+      case 3: left_apply<3>(m, z[i & 1], cur.tm, cur.off); break;
+      default: {  // a phase of the outer bits alone
+        int none[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        left_apply<0>(m, z[i & 1], 0, none);
       }
-#pragma unroll
-      for (int l = 0; l < 8; l++)
-        if (l < d) m[row | off[l]][c] = y[l];
     }
+    cur = nxt;
   }
   __syncthreads();
   // one 16-byte row of a core matrix at a time
