@@ -122,19 +122,32 @@ qs_status resolve_records(qs_state *st, bool wait) {
 
 qs_status fold_records(qs_state *st, bool wait) { return resolve_records(st, wait); }
 
-// Undoes the relabelling with physical bit exchanges (one per cycle step),
-// leaving perm = identity.
+// Undoes the relabelling with physical bit exchanges, leaving perm =
+// identity. Bit perm[l] has to move to position l: every cycle of that map,
+// c_i -> c_(i+1), is two reflections, c_i <-> c_(-i) and then c_i <-> c_(1-i)
+// (indices modulo its length), so two sets of disjoint exchanges do it.
 cudaError_t to_logical_order(qs_state *st) {
-  for (int l = 0; l < st->n; l++) {
-    if (st->perm[l] == l) continue;
-    int other = -1;
-    for (int k = 0; k < st->n; k++)
-      if (st->perm[k] == l) other = k;
-    cudaError_t e = launch_permute(st->amps, st->n, st->dtype == QS_C128, st->perm[l], l, st->stream);
-    if (e != cudaSuccess) return e;
-    st->perm[other] = st->perm[l];
-    st->perm[l] = (int8_t)l;
+  int next[QS_MAX_QUBITS];
+  for (int l = 0; l < st->n; l++) next[st->perm[l]] = l;
+  std::vector<std::pair<int, int>> first, second;
+  bool seen[QS_MAX_QUBITS] = {false};
+  for (int q = 0; q < st->n; q++) {
+    std::vector<int> c;
+    for (int x = q; !seen[x]; x = next[x]) {
+      seen[x] = true;
+      c.push_back(x);
+    }
+    const int len = (int)c.size();
+    for (int i = 0; i < len; i++) {
+      const int r1 = (len - i) % len, r2 = (len + 1 - i) % len;
+      if (i < r1) first.push_back({std::min(c[i], c[r1]), std::max(c[i], c[r1])});
+      if (i < r2) second.push_back({std::min(c[i], c[r2]), std::max(c[i], c[r2])});
+    }
   }
+  cudaError_t e = launch_bit_swaps(st->amps, st->n, st->dtype == QS_C128, first, st->stream);
+  if (e == cudaSuccess) e = launch_bit_swaps(st->amps, st->n, st->dtype == QS_C128, second, st->stream);
+  if (e != cudaSuccess) return e;
+  for (int l = 0; l < st->n; l++) st->perm[l] = (int8_t)l;
   return cudaSuccess;
 }
 

@@ -235,6 +235,9 @@ constexpr int kResidentBits = 13;
 bool resident_applies(const std::vector<Block> &plan, int n);
 cudaError_t run_resident(void *amps, int n, const std::vector<Block> &plan, cudaStream_t s);
 cudaError_t launch_permute(void *amps, int n, bool c128, int a, int b, cudaStream_t s);
+// Disjoint exchanges of physical bits, all at once.
+cudaError_t launch_bit_swaps(void *amps, int n, bool c128, const std::vector<std::pair<int, int>> &swaps,
+                             cudaStream_t s);
 cudaError_t launch_set_basis(void *amps, int n, bool c128, uint64_t idx, cudaStream_t s);
 
 // Marginal probabilities over m physical bits pos[0..m) (bin bit j = pos[j]).
