@@ -337,9 +337,64 @@ __global__ void __launch_bounds__(kT) k_fit(const __grid_constant__ FitParam P) 
   }
 }
 
+// Means and standard deviations of the features, then of the targets.
+struct Scaling {
+  float mean[kF + 1], std[kF + 1];
+};
+
+// FP64 mean and deviation of column blockIdx.x of n rows of kF features, or of
+// the targets (the last block). The FP64 rate (three operations a value, two
+// per clock) bounds it: 10 us for 10,000 rows, which the host took 250 us for.
+__global__ void __launch_bounds__(kT) k_scaling(const float *__restrict__ x, const float *__restrict__ t, int n,
+                                                float *__restrict__ out) {
+  __shared__ double part[kT];
+  const int f = blockIdx.x, tid = threadIdx.x;
+  const float *col = f < kF ? x + f : t;
+  const int step = f < kF ? kF : 1;
+  auto total = [&](double v) {
+    part[tid] = v;
+    __syncthreads();
+    for (int o = kT / 2; o > 0; o >>= 1) {
+      if (tid < o) part[tid] += part[tid + o];
+      __syncthreads();
+    }
+    const double s = part[0];
+    __syncthreads();
+    return s;
+  };
+  double s = 0;
+  for (int r = tid; r < n; r += kT) s += (double)col[(size_t)r * step];
+  const double mean = total(s) / n;
+  s = 0;
+  for (int r = tid; r < n; r += kT) {
+    const double d = (double)col[(size_t)r * step] - mean;
+    s = fma(d, d, s);
+  }
+  const double var = total(s) / n;
+  if (tid == 0) {
+    out[f] = (float)mean;
+    // a feature counts as constant below 1e-6, the targets below a variance of 1e-12
+    out[kF + 1 + f] = (f < kF ? sqrt(var) > 1e-6 : var > 1e-12) ? (float)sqrt(var) : 1.f;
+  }
+}
+
+// Standardises n rows and their targets in place.
+__global__ void __launch_bounds__(kT) k_standardise(float *__restrict__ x, float *__restrict__ t, int n,
+                                                    const __grid_constant__ Scaling sc) {
+  const long long all = (long long)n * kF;
+  for (long long e = (long long)blockIdx.x * kT + threadIdx.x; e < all + n; e += (long long)gridDim.x * kT) {
+    if (e < all) {
+      const int f = (int)(e % kF);
+      x[e] = (x[e] - sc.mean[f]) / sc.std[f];
+    } else {
+      t[e - all] = (t[e - all] - sc.mean[kF]) / sc.std[kF];
+    }
+  }
+}
+
 // y[r] of n feature rows, 16 rows per tile.
 __global__ void __launch_bounds__(kT) k_predict(const float *__restrict__ x, const float *__restrict__ p,
-                                                float *__restrict__ y, int n) {
+                                                float *__restrict__ y, int n, const __grid_constant__ Scaling sc) {
   extern __shared__ __align__(16) unsigned char smem[];
   Weights &W = *reinterpret_cast<Weights *>(smem);
   Tile &T = *reinterpret_cast<Tile *>(smem + sizeof(Weights));
@@ -347,11 +402,11 @@ __global__ void __launch_bounds__(kT) k_predict(const float *__restrict__ x, con
   for (int i = tid; i < kParams; i += kT) reinterpret_cast<float *>(&W)[weight_slot(i)] = p[i];
   for (long long r0 = (long long)blockIdx.x * kS; r0 < n; r0 += (long long)gridDim.x * kS) {
     const int have = (int)min((long long)kS, n - r0);
-    for (int e = tid; e < kS * kF; e += kT) T.x[e] = e / kF < have ? x[r0 * kF + e] : 0.f;
+    for (int e = tid; e < kS * kF; e += kT) T.x[e] = e / kF < have ? (x[r0 * kF + e] - sc.mean[e % kF]) / sc.std[e % kF] : 0.f;
     __syncthreads();
     tile_forward(W, T);
     __syncthreads();
-    if (tid < have) y[r0 + tid] = T.y[tid];
+    if (tid < have) y[r0 + tid] = T.y[tid] * sc.std[kF] + sc.mean[kF];
   }
 }
 
@@ -363,8 +418,7 @@ struct qs_mlp {
   int *idx = nullptr;    // sample order
   int cap = 0;           // rows x, y, loss and idx hold
   int step = 0;
-  float x_mean[kF], x_std[kF], y_mean = 0.f, y_std = 1.f;
-  bool normalised = false;
+  Scaling scaling;
   cudaStream_t stream = nullptr;
 };
 
@@ -430,13 +484,9 @@ cudaError_t launch_fit(const FitParam &P, cudaStream_t s) {
 
 cudaError_t launch_predict(qs_mlp *mm, int n) {
   const int tiles = (n + kS - 1) / kS;
-  k_predict<<<std::min(tiles, 4 * qs::dev_info().sms), kT, kPredictSmem, mm->stream>>>(mm->x, mm->p, mm->y, n);
+  k_predict<<<std::min(tiles, 4 * qs::dev_info().sms), kT, kPredictSmem, mm->stream>>>(mm->x, mm->p, mm->y, n,
+                                                                                       mm->scaling);
   return cudaGetLastError();
-}
-
-void standardise(const qs_mlp *mm, const float *x, float *out, int n) {
-  for (int r = 0; r < n; r++)
-    for (int f = 0; f < kF; f++) out[(size_t)r * kF + f] = (x[(size_t)r * kF + f] - mm->x_mean[f]) / mm->x_std[f];
 }
 
 }  // namespace
@@ -449,9 +499,9 @@ qs_status qs_mlp_create(uint64_t seed, void *cuda_stream, qs_mlp **out) {
   qs_mlp *mm = new (std::nothrow) qs_mlp();
   if (!mm) return mfail(QS_ENOMEM, "qs_mlp_create: host allocation failed");
   mm->stream = (cudaStream_t)cuda_stream;
-  for (int f = 0; f < kF; f++) {
-    mm->x_mean[f] = 0.f;
-    mm->x_std[f] = 1.f;
+  for (int f = 0; f <= kF; f++) {
+    mm->scaling.mean[f] = 0.f;
+    mm->scaling.std[f] = 1.f;
   }
   // He-uniform initial weights, zero biases, from a seeded generator
   std::vector<float> p(kParams, 0.f);
@@ -525,45 +575,35 @@ qs_status qs_mlp_gradient(qs_mlp *mm, const float *x, const float *y, int n, flo
 qs_status qs_mlp_train(qs_mlp *mm, const float *x, const float *y, int n, int epochs, int batch, float lr,
                        uint64_t seed, float *loss_out) {
   if (!mm || !x || !y || n <= 0 || epochs <= 0 || batch <= 0) return mfail(QS_EINVAL, "qs_mlp_train: bad arguments");
-  // standardisation from this training set (features and targets)
-  std::vector<double> mu(kF, 0.0), var(kF, 0.0);
-  double ym = 0, yv = 0;
-  for (int r = 0; r < n; r++) {
-    for (int f = 0; f < kF; f++) mu[f] += x[(size_t)r * kF + f];
-    ym += y[r];
-  }
-  for (int f = 0; f < kF; f++) mu[f] /= n;
-  ym /= n;
-  for (int r = 0; r < n; r++) {
-    for (int f = 0; f < kF; f++) {
-      const double d = x[(size_t)r * kF + f] - mu[f];
-      var[f] += d * d;
-    }
-    yv += (y[r] - ym) * (y[r] - ym);
-  }
-  for (int f = 0; f < kF; f++) {
-    mm->x_mean[f] = (float)mu[f];
-    const double sd = std::sqrt(var[f] / n);
-    mm->x_std[f] = sd > 1e-6 ? (float)sd : 1.f;
-  }
-  mm->y_mean = (float)ym;
-  mm->y_std = yv / n > 1e-12 ? (float)std::sqrt(yv / n) : 1.f;
-  mm->normalised = true;
-  std::vector<float> xs((size_t)n * kF), ys(n);
-  standardise(mm, x, xs.data(), n);
-  for (int r = 0; r < n; r++) ys[r] = (y[r] - mm->y_mean) / mm->y_std;
+  // standardisation from this training set (features and targets), while the host draws the first order
+  static_assert(sizeof(Scaling) <= sizeof(float) * kParams, "the gradient's space holds it meanwhile");
   const int B = std::min(batch, n), steps = n / B;
   cudaError_t e = ensure_rows(mm, n);
-  if (e == cudaSuccess) e = cudaMemcpy(mm->x, xs.data(), sizeof(float) * xs.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(mm->y, ys.data(), sizeof(float) * n, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(mm->x, x, sizeof(float) * (size_t)n * kF, cudaMemcpyHostToDevice, mm->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(mm->y, y, sizeof(float) * (size_t)n, cudaMemcpyHostToDevice, mm->stream);
+  if (e == cudaSuccess) {
+    k_scaling<<<kF + 1, kT, 0, mm->stream>>>(mm->x, mm->y, n, mm->g);
+    e = cudaGetLastError();
+  }
   if (e != cudaSuccess) return mfail(QS_ECUDA, std::string("qs_mlp_train: ") + cudaGetErrorString(e));
   std::vector<int> order(n);
   for (int i = 0; i < n; i++) order[i] = i;
   std::mt19937_64 rng(seed);
+  std::shuffle(order.begin(), order.end(), rng);
+  Scaling sc;
+  e = cudaMemcpyAsync(&sc, mm->g, sizeof(sc), cudaMemcpyDeviceToHost, mm->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(mm->stream);
+  if (e == cudaSuccess) {
+    mm->scaling = sc;
+    const long long all = (long long)n * (kF + 1);
+    k_standardise<<<(int)std::min<long long>((all + kT - 1) / kT, 8ll * qs::dev_info().sms), kT, 0, mm->stream>>>(
+        mm->x, mm->y, n, sc);
+    e = cudaGetLastError();
+  }
   std::vector<float> lpart(B);
   double last = 0;
   for (int ep = 0; ep < epochs && e == cudaSuccess; ep++) {
-    std::shuffle(order.begin(), order.end(), rng);  // while the epoch before runs
+    if (ep > 0) std::shuffle(order.begin(), order.end(), rng);  // while the epoch before runs
     // one upload of the epoch's sample order, after the epoch before has read its own; the host buffer is
     // only reused after the stream has consumed it
     e = cudaMemcpyAsync(mm->idx, order.data(), sizeof(int) * n, cudaMemcpyHostToDevice, mm->stream);
@@ -590,15 +630,12 @@ qs_status qs_mlp_train(qs_mlp *mm, const float *x, const float *y, int n, int ep
 qs_status qs_mlp_predict(qs_mlp *mm, const float *x, int n, float *y_out) {
   if (!mm || !x || !y_out || n < 0) return mfail(QS_EINVAL, "qs_mlp_predict: bad arguments");
   if (n == 0) return QS_OK;
-  std::vector<float> xs((size_t)n * kF);
-  standardise(mm, x, xs.data(), n);
   cudaError_t e = ensure_rows(mm, n);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(mm->x, xs.data(), sizeof(float) * xs.size(), cudaMemcpyHostToDevice, mm->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(mm->x, x, sizeof(float) * (size_t)n * kF, cudaMemcpyHostToDevice, mm->stream);
   if (e == cudaSuccess) e = launch_predict(mm, n);
   if (e == cudaSuccess) e = cudaMemcpyAsync(y_out, mm->y, sizeof(float) * n, cudaMemcpyDeviceToHost, mm->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(mm->stream);
   if (e != cudaSuccess) return mfail(QS_ECUDA, std::string("qs_mlp_predict: ") + cudaGetErrorString(e));
-  for (int i = 0; i < n; i++) y_out[i] = y_out[i] * mm->y_std + mm->y_mean;
   return QS_OK;
 }
 
