@@ -61,43 +61,62 @@ __device__ __forceinline__ uint32_t rec_insert(uint32_t j, const RecHead &h) {
   return j;
 }
 
-// One thread per group; the matrix is read from shared memory two entries at
-// a time, the same address for the whole warp.
-template <int K> __device__ __forceinline__ void rec_dense(float2 *a, int n, const RecHead &h, const float4 *m) {
+// One thread per G groups, blockDim.x apart from first; the matrix is read from
+// shared memory two entries at a time, the same address for the whole warp.
+// Those reads bound a mat-vec of one group, so two groups share them where
+// there are that many (a batch of 192 QAOA circuits 3.37 -> 2.97 ms a run).
+// Four groups, with two CTAs per SM instead of three: 3.03 ms. Entries kept as
+// (x, x, -y, y) for packed multiply-adds, twice the words, 3.58 ms.
+template <int K, int G>
+__device__ __forceinline__ void rec_dense_groups(float2 *a, const RecHead &h, const float4 *m, uint32_t first) {
   constexpr int D = 1 << K;
   uint32_t d[K];
 #pragma unroll
   for (int j = 0; j < K; j++) d[j] = 1u << h.tq[j];
-  const uint32_t groups = 1u << (n - h.nf);
-  for (uint32_t g = threadIdx.x; g < groups; g += blockDim.x) {
-    float2 *p = a + (rec_insert(g, h) | h.cmask);
-    float2 v[D];
+  auto off = [&](int s) {
+    uint32_t o = 0;
 #pragma unroll
-    for (int s = 0; s < D; s++) {
-      uint32_t off = 0;
+    for (int j = 0; j < K; j++)
+      if ((s >> j) & 1) o += d[j];
+    return o;
+  };
+  float2 *p[G];
+  float2 v[G][D];
 #pragma unroll
-      for (int j = 0; j < K; j++)
-        if ((s >> j) & 1) off += d[j];
-      v[s] = p[off];
-    }
+  for (int g = 0; g < G; g++) {
+    p[g] = a + (rec_insert(first + g * blockDim.x, h) | h.cmask);
 #pragma unroll
-    for (int r = 0; r < D; r++) {
-      float re0 = 0.f, im0 = 0.f, re1 = 0.f, im1 = 0.f;
-#pragma unroll
-      for (int c = 0; c < D; c += 2) {
-        const float4 w = m[r * (D / 2) + c / 2];
-        re0 = fmaf(w.x, v[c].x, fmaf(-w.y, v[c].y, re0));
-        im0 = fmaf(w.x, v[c].y, fmaf(w.y, v[c].x, im0));
-        re1 = fmaf(w.z, v[c + 1].x, fmaf(-w.w, v[c + 1].y, re1));
-        im1 = fmaf(w.z, v[c + 1].y, fmaf(w.w, v[c + 1].x, im1));
-      }
-      uint32_t off = 0;
-#pragma unroll
-      for (int j = 0; j < K; j++)
-        if ((r >> j) & 1) off += d[j];
-      p[off] = make_float2(re0 + re1, im0 + im1);
-    }
+    for (int s = 0; s < D; s++) v[g][s] = p[g][off(s)];
   }
+#pragma unroll
+  for (int r = 0; r < D; r++) {
+    float re0[G], im0[G], re1[G], im1[G];
+#pragma unroll
+    for (int g = 0; g < G; g++) re0[g] = im0[g] = re1[g] = im1[g] = 0.f;
+#pragma unroll
+    for (int c = 0; c < D; c += 2) {
+      const float4 w = m[r * (D / 2) + c / 2];
+#pragma unroll
+      for (int g = 0; g < G; g++) {
+        re0[g] = fmaf(w.x, v[g][c].x, fmaf(-w.y, v[g][c].y, re0[g]));
+        im0[g] = fmaf(w.x, v[g][c].y, fmaf(w.y, v[g][c].x, im0[g]));
+        re1[g] = fmaf(w.z, v[g][c + 1].x, fmaf(-w.w, v[g][c + 1].y, re1[g]));
+        im1[g] = fmaf(w.z, v[g][c + 1].y, fmaf(w.w, v[g][c + 1].x, im1[g]));
+      }
+    }
+#pragma unroll
+    for (int g = 0; g < G; g++) p[g][off(r)] = make_float2(re0[g] + re1[g], im0[g] + im1[g]);
+  }
+}
+
+template <int K> __device__ __forceinline__ void rec_dense(float2 *a, int n, const RecHead &h, const float4 *m) {
+  const uint32_t groups = 1u << (n - h.nf);
+  if (K <= 3 && groups >= 2 * blockDim.x) {  // powers of two: whole pairs
+    if constexpr (K <= 3)
+      for (uint32_t g = threadIdx.x; g < groups; g += 2 * blockDim.x) rec_dense_groups<K, 2>(a, h, m, g);
+    return;
+  }
+  for (uint32_t g = threadIdx.x; g < groups; g += blockDim.x) rec_dense_groups<K, 1>(a, h, m, g);
 }
 
 __device__ __forceinline__ float2 rec_cmul(float2 w, float2 v) {
@@ -182,7 +201,8 @@ __device__ __forceinline__ void tile_phase(const uint32_t *w, int nb, int m, con
 
 // Applies one record; ends with the CTA synchronised. MAXT bounds the
 // registers: the 5- and 6-target mat-vecs exist where it is at most 256.
-// TILE: a is a tile over the n bits tile_q, at base in the state.
+// TILE: a is a tile over the n bits tile_q, at base in the state; its blocks
+// have at most four targets.
 template <int MAXT, bool TILE = false>
 __device__ __forceinline__ void rec_apply(float2 *a, int n, const uint4 *rec, uint32_t base = 0,
                                           const int *tile_q = nullptr, RecPhase *scratch = nullptr) {
@@ -197,10 +217,10 @@ __device__ __forceinline__ void rec_apply(float2 *a, int n, const uint4 *rec, ui
       case 3: rec_dense<3>(a, n, h, m); break;
       case 4: rec_dense<4>(a, n, h, m); break;
       case 5:
-        if constexpr (MAXT <= 256) rec_dense<5>(a, n, h, m);
+        if constexpr (MAXT <= 256 && !TILE) rec_dense<5>(a, n, h, m);
         break;
       case 6:
-        if constexpr (MAXT <= 256) rec_dense<6>(a, n, h, m);
+        if constexpr (MAXT <= 256 && !TILE) rec_dense<6>(a, n, h, m);
         break;
       default: break;
     }
