@@ -135,7 +135,10 @@ __device__ __forceinline__ float2 turn(uint32_t p) {
 }
 
 // A thread's amplitudes differ only in the bits above the thread index: the
-// terms among and with the lower bits are summed once.
+// terms among and with the lower bits are summed once, those of the bits above
+// the lowest three of them once for eight amplitudes. (Summed anew for each
+// amplitude, these integer additions took as many issue slots as all else that
+// a batch's tile kernel does.)
 __device__ __forceinline__ void rec_phase(float2 *a, int n, const RecPhase &ph) {
   const int tb = 31 - __clz(blockDim.x);  // a power of two of threads
   const uint32_t t = threadIdx.x;
@@ -155,16 +158,32 @@ __device__ __forceinline__ void rec_phase(float2 *a, int n, const RecPhase &ph) 
       for (int l = 0; l < tb; l++)
         if ((t >> l) & 1) up[i] += ph.b[tb + i][l];
     }
-  for (uint32_t x = t, j = 0; x < (1u << n); x += blockDim.x, j++) {
-    uint32_t phi = phi0;
+  uint32_t pair[3] = {0, 0, 0};  // among the lowest three: (1, 0), (2, 0), (2, 1)
+  if (tb + 1 < n) pair[0] = ph.b[tb + 1][tb];
+  if (tb + 2 < n) pair[1] = ph.b[tb + 2][tb], pair[2] = ph.b[tb + 2][tb + 1];
+  const uint32_t all = 1u << n;
+  for (uint32_t j = 0; 8 * j * blockDim.x < all; j++) {
+    uint32_t base = phi0, u[3] = {up[0], up[1], up[2]};
 #pragma unroll
-    for (int i = 0; i < 6; i++)
-      if ((j >> i) & 1) {
-        phi += up[i];
+    for (int i = 0; i < 3; i++)
+      if ((j >> i) & 1) {  // bit tb + 3 + i is set
+        const uint32_t *row = ph.b[tb + 3 + i] + tb;
+        base += up[3 + i];
+#pragma unroll
+        for (int l = 0; l < 3; l++) u[l] += row[l];
+#pragma unroll
         for (int l = 0; l < i; l++)
-          if ((j >> l) & 1) phi += ph.b[tb + i][tb + l];
+          if ((j >> l) & 1) base += row[3 + l];
       }
-    a[x] = rec_cmul(turn(phi), a[x]);
+#pragma unroll
+    for (uint32_t e = 0; e < 8; e++) {
+      const uint32_t x = t + (8 * j + e) * blockDim.x;
+      uint32_t phi = base;
+      if (e & 1) phi += u[0];
+      if (e & 2) phi += u[1] + ((e & 1) ? pair[0] : 0u);
+      if (e & 4) phi += u[2] + ((e & 1) ? pair[1] : 0u) + ((e & 2) ? pair[2] : 0u);
+      if (x < all) a[x] = rec_cmul(turn(phi), a[x]);
+    }
   }
 }
 
