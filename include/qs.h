@@ -207,8 +207,11 @@ qs_status qs_parse_qasm(const char *text, int *n_qubits, qs_gate *gates, size_t 
  * gates fused again, at most opts->tile_k wide -- in shared memory during one
  * read and one write of the state (QS_TILE is ignored when n <= tile bits);
  * QS_PGO_RULES / QS_PGO_MEASURED replace the pass flags by the activator's
- * choice (see qs_pgo_select). gates is copied during the call; the launches
- * are asynchronous on the state's stream.
+ * choice (see qs_pgo_select). Under QS_PGO_RULES, without QS_PROFILE, dense
+ * complex64 circuits of more than 13 qubits may run as tile passes on the
+ * tensor cores: several 5-target blocks per read and write of the state.
+ * gates is copied during the call; the launches are asynchronous on the
+ * state's stream.
  */
 qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, uint64_t flags,
                            const qs_opts *opts);
@@ -245,8 +248,9 @@ typedef struct {
   double t_start_ms; /* start relative to the first block (QS_PROFILE), else -1 */
   double ms;         /* device time (QS_PROFILE), else -1 */
   int64_t tiles;     /* blocks of an apply call: tensor-core blocks, tiles of 128 groups;
-                        phase polynomials, chunks of 1024 amplitudes; else 0 (also where a
-                        narrow state's blocks share one launch) */
+                        phase polynomials, chunks of 1024 amplitudes; tensor-core tile passes,
+                        tiles of 4096 amplitudes; else 0 (also where a narrow state's blocks
+                        share one launch) */
   int32_t ctas;      /* the same blocks: CTAs launched (each loops over tiles ctas apart;
                         each of a phase CTA's 8 warps over chunks 8 ctas apart); else 0 */
   int32_t reserved;

@@ -345,7 +345,7 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
     if (!tiles) break;
     // their operands take more device memory than single blocks': without it
     // the call runs block by block
-    size_t need = operand_program_bytes(plan);
+    size_t need = (operand_program_bytes(plan) + 255) & ~(size_t)255;
     for (const Block &b : plan) need += dev_operand_bytes(b) + ((block_dev_matrix_bytes(b, c128) + 255) & ~(size_t)255);
     unsigned char *dm = (unsigned char *)st->d_mats;
     if (grow(dm, st->mats_cap, need) == cudaSuccess) {
