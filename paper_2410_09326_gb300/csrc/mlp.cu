@@ -446,6 +446,13 @@ cudaError_t ensure_rows(qs_mlp *mm, int n) {
   return e;
 }
 
+// All of a model's work is ordered on its stream, which need not wait for the
+// legacy stream; the host buffer is free again on return.
+cudaError_t copy(qs_mlp *mm, void *dst, const void *src, size_t bytes, cudaMemcpyKind kind) {
+  cudaError_t e = cudaMemcpyAsync(dst, src, bytes, kind, mm->stream);
+  return e == cudaSuccess ? cudaStreamSynchronize(mm->stream) : e;
+}
+
 constexpr size_t kFitSmem = sizeof(Weights) + sizeof(Tile) + sizeof(float) * kParams;
 constexpr size_t kPredictSmem = sizeof(Weights) + sizeof(Tile);
 
@@ -519,9 +526,9 @@ qs_status qs_mlp_create(uint64_t seed, void *cuda_stream, qs_mlp **out) {
     mm->g = mm->p + kParams;
     mm->m = mm->g + kParams;
     mm->v = mm->m + kParams;
-    e = cudaMemcpy(mm->p, p.data(), sizeof(float) * kParams, cudaMemcpyHostToDevice);
+    e = cudaMemsetAsync(mm->m, 0, 2 * sizeof(float) * kParams, mm->stream);
   }
-  if (e == cudaSuccess) e = cudaMemset(mm->m, 0, 2 * sizeof(float) * kParams);
+  if (e == cudaSuccess) e = copy(mm, mm->p, p.data(), sizeof(float) * kParams, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     qs_mlp_free(mm);
     return mfail(QS_ENOMEM, std::string("qs_mlp_create: ") + cudaGetErrorString(e));
@@ -544,8 +551,8 @@ void qs_mlp_free(qs_mlp *mm) {
 qs_status qs_mlp_params(qs_mlp *mm, float *host_out, const float *host_in) {
   if (!mm) return mfail(QS_EINVAL, "qs_mlp_params: null model");
   cudaError_t e = cudaSuccess;
-  if (host_in) e = cudaMemcpy(mm->p, host_in, sizeof(float) * kParams, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && host_out) e = cudaMemcpy(host_out, mm->p, sizeof(float) * kParams, cudaMemcpyDeviceToHost);
+  if (host_in) e = copy(mm, mm->p, host_in, sizeof(float) * kParams, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && host_out) e = copy(mm, host_out, mm->p, sizeof(float) * kParams, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return mfail(QS_ECUDA, std::string("qs_mlp_params: ") + cudaGetErrorString(e));
   return QS_OK;
 }
@@ -553,17 +560,16 @@ qs_status qs_mlp_params(qs_mlp *mm, float *host_out, const float *host_in) {
 qs_status qs_mlp_gradient(qs_mlp *mm, const float *x, const float *y, int n, float *grad_out, float *loss_out) {
   if (!mm || !x || !y || n <= 0 || !grad_out) return mfail(QS_EINVAL, "qs_mlp_gradient: bad arguments");
   cudaError_t e = ensure_rows(mm, n);
-  if (e == cudaSuccess) e = cudaMemcpy(mm->x, x, sizeof(float) * (size_t)n * kF, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(mm->y, y, sizeof(float) * (size_t)n, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(mm->x, x, sizeof(float) * (size_t)n * kF, cudaMemcpyHostToDevice, mm->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(mm->y, y, sizeof(float) * (size_t)n, cudaMemcpyHostToDevice, mm->stream);
   if (e == cudaSuccess) {
     FitParam P = {mm->x, mm->y, nullptr, mm->p, mm->g, mm->m, mm->v, mm->loss, n, 1, 0, 0, 0.f};
     e = launch_fit(P, mm->stream);
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(mm->stream);
-  if (e == cudaSuccess) e = cudaMemcpy(grad_out, mm->g, sizeof(float) * kParams, cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = copy(mm, grad_out, mm->g, sizeof(float) * kParams, cudaMemcpyDeviceToHost);
   if (e == cudaSuccess && loss_out) {
     std::vector<float> l(n);
-    e = cudaMemcpy(l.data(), mm->loss, sizeof(float) * n, cudaMemcpyDeviceToHost);
+    e = copy(mm, l.data(), mm->loss, sizeof(float) * n, cudaMemcpyDeviceToHost);
     double s = 0;
     for (float v : l) s += v;
     *loss_out = (float)(s / n);
