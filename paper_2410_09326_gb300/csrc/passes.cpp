@@ -656,8 +656,10 @@ qs_status tile_plan(int n, const std::vector<qs_gate> &pg, const std::vector<int
 // Cost of a tile pass of b blocks, in launches of a single block of up to five
 // targets. Measured 0.45 + 0.4 b: at 27 qubits, where a block is an HBM pass,
 // 80 for the 30-qubit random circuit's 45 passes with 151 blocks (125 blocks
-// one by one), and as much at 19 qubits, where launches and latency count.
-double tc_tile_cost(size_t b) { return 0.45 + 0.4 * (double)b; }
+// one by one), and as much at 19 qubits, where launches and latency count. A
+// lone block gains nothing from a tile: three targets at 26 qubits 341 us with
+// the call's host time, 323 us by itself, at 16 qubits 91 and 30 us.
+double tc_tile_cost(size_t b) { return b == 1 ? 1.0 : 0.45 + 0.4 * (double)b; }
 
 // Tensor-core tile passes (tc_tile.cu): gates grouped as in tile_plan into
 // passes whose non-diagonal qubits fit a tile of kTcTileBits, each pass's gates into
@@ -693,8 +695,9 @@ std::vector<int> one_qubit_late(const std::vector<qs_gate> &pg, const std::vecto
   return out;
 }
 
-// A pass whose gates cost less as blocks of K qubits one by one stays that.
-// Returns the pass's cost. search: blocks by first fit or by roll-outs,
+// A pass whose gates cost less as blocks of K qubits one by one stays that, as
+// does one that has no block of four qubits: those run in FP32 (0.75e-7 off a
+// block of three targets, a tile's members 1.1e-7). Returns the pass's cost. search: blocks by first fit or by roll-outs,
 // whichever are fewer.
 double tc_tile_blocks(int n, const std::vector<qs_gate> &pg, const Pending &pass, int K, bool search, TcPass &out) {
   uint64_t t = pass.tmask | ((1ull << kTileLowBits) - 1);
@@ -715,7 +718,9 @@ double tc_tile_blocks(int n, const std::vector<qs_gate> &pg, const Pending &pass
   greedy_groups(pg, idx, single, [&](const Pending &p, int, uint64_t gmask, uint64_t, bool) {
     return popcount64(p.qmask | gmask) <= K;
   });
-  if ((double)single.size() <= tc_tile_cost(out.blocks.size())) {
+  bool fp32 = true;
+  for (const Pending &p : single) fp32 = fp32 && popcount64(p.qmask) < 4;
+  if (fp32 || (double)single.size() <= tc_tile_cost(out.blocks.size())) {
     out.single = true;
     out.blocks.swap(single);
     return (double)out.blocks.size();

@@ -150,6 +150,32 @@ def test_profiled_calls_scarce_memory_and_explicit_flags_run_block_by_block():
     assert not any(r.kind == 3 for r in recs)
 
 
+@pytest.mark.parametrize("t", [[5, 6, 7], [1, 8, 14], [0, 3, 4, 9, 12]])
+def test_a_lone_block_runs_by_itself(t):
+    """A tile pass pays for several blocks."""
+    n, r, gates = 16, random.Random(4), []
+    for _ in range(3):
+        gates += [("u3", [q], [r.uniform(0, 6.28) for _ in range(3)]) for q in t]
+        gates += [("cx", [a, b]) for a, b in zip(t, t[1:])]
+    init = _random_state(n, 6)
+    got, recs = _run(n, gates, init)
+    assert [(r.k, r.tc > 0) for r in recs if r.kind == 0] == [(len(t), len(t) > 3)]
+    assert not any(r.kind == 3 for r in recs)
+    want, _ = oracle.simulate(cg.to_qasm(n, gates), init=init.astype(np.complex64).astype(np.complex128))
+    assert np.linalg.norm(got - want) <= 2.5e-7
+
+
+def test_blocks_of_up_to_three_targets_keep_their_fp32_arithmetic():
+    n = 16
+    init = _random_state(n, 6)
+    got, recs = _run(n, [("ccx", [0, 5, 9]), ("ccx", [13, 2, 4]), ("ccx", [7, 8, 12])], init)
+    assert [(r.kind, r.k, r.nctrl, r.tc) for r in recs if r.kind != 2] == [(0, 1, 2, 0)] * 3
+    x = np.arange(1 << n)
+    for a, b, t in ((7, 8, 12), (13, 2, 4), (0, 5, 9)):
+        x ^= ((x >> a) & (x >> b) & 1) << t
+    assert np.array_equal(got.astype(np.complex64), init.astype(np.complex64)[x])
+
+
 def test_timeout_is_reported():
     n = 14
     gates = qs.gates_to_array(_layers(n, 3, 1, ["cx"]))
