@@ -561,6 +561,10 @@ __global__ void __launch_bounds__(256) k_probs_chunk(const T *__restrict__ a, co
     for (int k = 0; k < SLOTS; k++)
       if (p.lo_pos[i] == slot_bit(k)) slot_sub[k] = 1 << i;
   }
+  unsigned gone = 0;  // slot bits a flush sums over
+#pragma unroll
+  for (int k = 0; k < SLOTS; k++) gone |= (~measured >> slot_bit(k) & 1u) << k;
+  const unsigned lanes = ~measured >> LANE0 & 31u;  // and lane bits
   auto lo_bin = [&](int s) {
     unsigned b = 0;
     for (int i = 0; i < p.m_lo; i++) b |= (unsigned)((s >> i) & 1) << p.lo_j[i];
@@ -589,32 +593,34 @@ __global__ void __launch_bounds__(256) k_probs_chunk(const T *__restrict__ a, co
       v[e] = (double)acc[e] - (double)comp[e];
       acc[e] = comp[e] = 0;
     }
-    unsigned gone = 0;  // slot bits summed over
+    // (the branches are the same for all threads, and real ones: adding along
+    // every slot and lane bit with a select took 10 us of FP64 time a flush)
+    if (gone == NSLOT - 1) {
 #pragma unroll
-    for (int k = 0; k < SLOTS; k++) {
-      if ((measured >> slot_bit(k)) & 1) continue;
+      for (int d = 1; d < NSLOT; d *= 2)
 #pragma unroll
-      for (int e = 0; e < NSLOT; e++)
-        if (!((e >> k) & 1) && (e & gone) == 0) v[e] += v[e | (1 << k)];
-      gone |= 1u << k;
-    }
-    unsigned lanes = 0;  // lane bits summed over
+        for (int e = 0; e < NSLOT; e += 2 * d) v[e] += v[e + d];
+    } else {
 #pragma unroll
-    for (int j = 0; j < 5; j++) {
-      if ((measured >> (LANE0 + j)) & 1) continue;
+      for (int k = 0; k < SLOTS; k++)
+        if ((gone >> k) & 1) {
 #pragma unroll
-      for (int e = 0; e < NSLOT; e++)
-        if ((e & gone) == 0) v[e] += __shfl_xor_sync(0xffffffffu, v[e], 1 << j);
-      lanes |= 1u << j;
+          for (int e = 0; e < NSLOT; e++)
+            if (!((e >> k) & 1)) v[e] += v[e | (1 << k)];
+        }
     }
 #pragma unroll
     for (int e = 0; e < NSLOT; e++) {
-      if ((e & gone) != 0 || (lane & lanes) != 0 || v[e] == 0.0) continue;
+      if ((e & gone) != 0) continue;
+      double x = v[e];
+#pragma unroll 1
+      for (unsigned r = lanes; r; r &= r - 1) x += __shfl_xor_sync(0xffffffffu, x, r & -r);
+      if ((lane & lanes) != 0 || x == 0.0) continue;
       int s = sub0;
 #pragma unroll
       for (int k = 0; k < SLOTS; k++)
         if ((e >> k) & 1) s |= slot_sub[k];
-      atomicAdd(&hist[s], v[e]);
+      atomicAdd(&hist[s], x);
     }
     __syncthreads();
     for (int s = threadIdx.x; s < nsub; s += blockDim.x) {
@@ -846,10 +852,14 @@ cudaError_t launch_probs(const void *amps, int n, bool c128, const int *pos, int
     c.n_chunks = 1ll << (n - kProbChunkBits);
     cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double) * (size_t)nb, s);
     if (e != cudaSuccess) return e;
-    // one wave of resident CTAs
+    // One wave of resident CTAs. A flush costs an SM 2 us of FP64 time for each
+    // of them (the sums' conversions and additions), so that more than two per
+    // SM pay only where they have chunks enough, and complex128 never: 24
+    // qubits and below took up to 1.4 times as long with three (22 qubits, the
+    // highest 8 measured: 46 -> 65 us), at 29 qubits three take 650 us, two 690.
     const int occ = c128 ? resident_ctas((const void *)k_probs_chunk<double2>, 256, 0)
                          : resident_ctas((const void *)k_probs_chunk<float2>, 256, 0);
-    long long grid = (long long)dev_info().sms * occ;
+    long long grid = (long long)dev_info().sms * std::min(occ, !c128 && n >= 25 ? 3 : 2);
     if (grid > c.n_chunks) grid = c.n_chunks;
     if (c128) k_probs_chunk<double2><<<(int)grid, 256, 0, s>>>((const double2 *)amps, c, out);
     else k_probs_chunk<float2><<<(int)grid, 256, 0, s>>>((const float2 *)amps, c, out);
