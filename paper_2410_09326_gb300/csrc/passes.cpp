@@ -111,12 +111,10 @@ template <typename F> void parallel_for(size_t n, double work_us, F f) {
   for (auto &x : th) x.join();
 }
 
-// f(0..n) for a handful of independent tasks, one host thread each.
-template <typename F> void run_tasks(size_t n, F f) {
-  std::vector<std::thread> th;
-  for (size_t i = 1; i < n; i++) th.emplace_back([&f, i] { f(i); });
-  if (n > 0) f(0);
-  for (auto &t : th) t.join();
+// As many gates of a long list as these cost roll-outs of `horizon` gates: a
+// short list's roll-outs end with it, and have fewer blocks to try.
+double roll_out_gates(size_t gates, int horizon) {
+  return (double)gates * std::min(1.0, (double)gates / (2.0 * (double)std::max(horizon, 1)));
 }
 
 struct Pending {
@@ -656,10 +654,8 @@ qs_status tile_plan(int n, const std::vector<qs_gate> &pg, const std::vector<int
 // Cost of a tile pass of b blocks, in launches of a single block of up to five
 // targets. Measured 0.45 + 0.4 b: at 27 qubits, where a block is an HBM pass,
 // 80 for the 30-qubit random circuit's 45 passes with 151 blocks (125 blocks
-// one by one), and as much at 19 qubits, where launches and latency count. A
-// lone block gains nothing from a tile: three targets at 26 qubits 341 us with
-// the call's host time, 323 us by itself, at 16 qubits 91 and 30 us.
-double tc_tile_cost(size_t b) { return b == 1 ? 1.0 : 0.45 + 0.4 * (double)b; }
+// one by one), and as much at 19 qubits, where launches and latency count.
+double tc_tile_cost(size_t b) { return 0.45 + 0.4 * (double)b; }
 
 // Tensor-core tile passes (tc_tile.cu): gates grouped as in tile_plan into
 // passes whose non-diagonal qubits fit a tile of kTcTileBits, each pass's gates into
@@ -760,7 +756,7 @@ double tc_tile_passes(int n, const std::vector<qs_gate> &pg, const std::vector<i
   const Variant variants[] = {{0, 0}, {60, 1}, {60, 2}, {40, 2}};
   std::vector<TcPass> alt[4];
   double total[4] = {0, 0, 0, 0};
-  run_tasks(4, [&](size_t v) {
+  parallel_for(4, 9.0 * roll_out_gates(all.size(), 60), [&](size_t v) {
     std::vector<Pending> passes;
     if (v == 0) {
       first_fit(passes);
@@ -881,14 +877,21 @@ qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<
     // 107 for the 30-qubit random circuit): from 27 qubits on (25).
     const int wide = n + (c128 ? 1 : 0);
     const bool search = opts.fuse_lookahead > 0 && (wide >= kSearchBits || repeated);
-    if (tc_tiles) {
-      tiled_cost = tc_tile_passes(n, pg, all, K, search, passes);
-      first_fit(groups);
+    first_fit(groups);
+    // (a circuit of one block gains nothing from a tile: three targets at 26
+    // qubits 341 us with the call's host time, 323 us by itself, at 16 qubits
+    // 91 and 30 us)
+    if (tc_tiles && groups.size() > 1) {
+      // Roll-outs cost by the gate and gain by the block: not where a block
+      // has many gates (all pairs of 26 qubits in one diagonal run, 325 gates,
+      // lost 0.5 ms to them). Layered circuits have 11 to 14 gates to a block.
+      const double block_gates = std::ldexp(16.0, n - (n < kPassSearchBits ? kSearchBits : kPassSearchBits));
+      const bool roll_outs = search && (double)all.size() <= block_gates * (double)groups.size();
+      tiled_cost = tc_tile_passes(n, pg, all, K, roll_outs, passes);
       // not searched where no search (it saves one block in six) would change the choice
       tiled_tc = tiled_cost < (search ? 0.8 : 1.0) * (double)groups.size();
-      if (!tiled_tc && search) groups.clear();
     }
-    if (search && !tiled_tc) {
+    if (search && !tiled_tc && groups.size() > 1) {
       // no horizon or tie-break (by the width of the last 6 or 12 blocks) is
       // best on every circuit: first fit and several roll-outs run side by
       // side on host threads, and the grouping with the fewest blocks is
@@ -904,21 +907,16 @@ qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<
       const size_t count = n + (c128 ? 2 : 0) >= kFullSearchBits ? 9 : 4;
       std::vector<std::vector<Pending>> alt(count);
       auto one = [&](size_t v) {
-        if (v == 0) first_fit(alt[0]);
+        if (v == 0) alt[0] = groups;
         else lookahead_groups(pg, all, alt[v], fits, variants[v].horizon, variants[v].tail, variants[v].free_joins);
       };
-      if (repeated) {  // many circuits are planned one after the other: threads would cost more than they save
-        for (size_t v = 0; v < count; v++) one(v);
-      } else {
-        run_tasks(count, one);
-      }
+      // (in batches many circuits are planned one after the other: threads would cost more than they save)
+      parallel_for(count, repeated ? 0 : (count > 4 ? 20.0 : 3.0) * roll_out_gates(all.size(), L), one);
       size_t best = 0;
       for (size_t v = 1; v < count; v++)
         if (alt[v].size() < alt[best].size()) best = v;
       groups.swap(alt[best]);
       tiled_tc = tc_tiles && tiled_cost < (double)groups.size();
-    } else if (!tc_tiles) {
-      first_fit(groups);
     }
   }
 
