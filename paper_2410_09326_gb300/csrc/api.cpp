@@ -345,7 +345,7 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
     if (!tiles) break;
     // their operands take more device memory than single blocks': without it
     // the call runs block by block
-    size_t need = (operand_program_bytes(plan) + 255) & ~(size_t)255;
+    size_t need = (operand_program_bytes(plan.data(), plan.size()) + 255) & ~(size_t)255;
     for (const Block &b : plan) need += dev_operand_bytes(b) + ((block_dev_matrix_bytes(b, c128) + 255) & ~(size_t)255);
     unsigned char *dm = (unsigned char *)st->d_mats;
     if (grow(dm, st->mats_cap, need) == cudaSuccess) {
@@ -362,27 +362,48 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
   // nor where each block is timed)
   const bool resident = !c128 && !prof && (flags & (QS_FUSE | QS_DIAG)) && o.threads == 0 && o.tc_max_ctas == 0 &&
                         resident_applies(plan, st->n);
-  // matrices of wide dense blocks: one pinned staging buffer, one copy
-  size_t mat_bytes = 0, operand_bytes = 0;
-  std::vector<size_t> mat_off(plan.size(), (size_t)-1);
+  // Device data: matrices, tables and the gates of tile passes as they are
+  // staged; then the operands of single tensor-core blocks, of which the
+  // matrices alone are staged (an eighth to a half of the operand) and spread
+  // over equal slots, k by k; then the operands of tile passes.
+  const size_t none = (size_t)-1;
+  std::vector<size_t> mat_off(plan.size(), none), host_off(plan.size(), none);
+  size_t up_bytes = 0;
   for (size_t i = 0; i < plan.size(); i++)
-    if (!resident && block_needs_dev_matrix(plan[i], c128)) {
-      mat_off[i] = mat_bytes;
-      mat_bytes += (block_dev_matrix_bytes(plan[i], c128) + 255) & ~(size_t)255;
+    if (!resident && block_needs_dev_matrix(plan[i], c128) && !made_on_device(plan[i])) {
+      mat_off[i] = host_off[i] = up_bytes;
+      up_bytes += (block_dev_matrix_bytes(plan[i], c128) + 255) & ~(size_t)255;
     }
-  // tensor-core tile passes: their gates in the same upload, the operands made
-  // from them behind it
-  const size_t prog_off = mat_bytes;
-  if (tiles) mat_bytes += (operand_program_bytes(plan) + 255) & ~(size_t)255;
+  const size_t prog_off = up_bytes;
+  if (tiles) up_bytes += (operand_program_bytes(plan.data(), plan.size()) + 255) & ~(size_t)255;
+  struct Slots {
+    size_t dev, host, slot, mat, count;
+  } slots[3];
+  size_t dev_bytes = up_bytes, host_bytes = up_bytes;
+  for (int k = 4; k <= 6; k++) {
+    Slots &x = slots[k - 4];
+    x = {dev_bytes, host_bytes, 0, 0, 0};
+    for (size_t i = 0; i < plan.size(); i++) {
+      if (resident || !made_on_device(plan[i]) || plan[i].k != k) continue;
+      x.slot = (block_dev_matrix_bytes(plan[i], c128) + 255) & ~(size_t)255;
+      x.mat = plan[i].mat.size() * (c128 ? 16 : 8);
+      mat_off[i] = x.dev + x.count * x.slot;
+      host_off[i] = x.host + x.count * x.mat;
+      x.count++;
+    }
+    dev_bytes += x.count * x.slot;
+    host_bytes += x.count * x.mat;
+  }
+  const size_t tile_off = dev_bytes;
   for (size_t i = 0; i < plan.size(); i++)
     if (const size_t ob = dev_operand_bytes(plan[i])) {
-      mat_off[i] = mat_bytes + operand_bytes;
-      operand_bytes += ob;
+      mat_off[i] = dev_bytes;
+      dev_bytes += ob;
     }
   bool any_tc = false;
   for (const Block &b : plan) any_tc |= b.tc;
   cudaError_t e;
-  if (mat_bytes) {
+  if (host_bytes) {
     if (st->mats_copied) {
       e = cudaEventSynchronize(st->mats_copied);  // staging buffer free again
       if (e != cudaSuccess) return cuda_fail(st, e, "qs_apply_circuit");
@@ -390,41 +411,35 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
       e = cudaEventCreateWithFlags(&st->mats_copied, cudaEventDisableTiming);
       if (e != cudaSuccess) return cuda_fail(st, e, "qs_apply_circuit");
     }
-    if (mat_bytes > st->h_mats_cap) {
+    if (host_bytes > st->h_mats_cap) {
       if (st->h_mats) cudaFreeHost(st->h_mats);
       st->h_mats = nullptr;
       st->h_mats_cap = 0;
-      e = cudaMallocHost(&st->h_mats, mat_bytes);
+      e = cudaMallocHost(&st->h_mats, host_bytes);
       if (e != cudaSuccess) return fail(QS_ENOMEM, "pinned staging allocation failed");
-      st->h_mats_cap = mat_bytes;
+      st->h_mats_cap = host_bytes;
     }
-    size_t cap_bytes = st->mats_cap;
     unsigned char *dm = (unsigned char *)st->d_mats;
-    if (mat_bytes + operand_bytes > cap_bytes) {
-      dev_free(dm);
-      dm = nullptr;
-      st->d_mats = nullptr;
-      st->mats_cap = 0;
-      e = dev_malloc((void **)&dm, mat_bytes + operand_bytes);
-      if (e != cudaSuccess) return fail(QS_ENOMEM, "matrix buffer allocation failed");
-      st->d_mats = dm;
-      st->mats_cap = mat_bytes + operand_bytes;
-    }
-    // (a phase polynomial's table takes about 30 us, a matrix 0.25 ns a byte of its operand)
-    double fill_us = 0.25e-3 * (double)mat_bytes;
+    e = grow(dm, st->mats_cap, dev_bytes);
+    st->d_mats = dm;
+    if (e != cudaSuccess) return fail(QS_ENOMEM, "matrix buffer allocation failed");
+    // (a phase polynomial's table takes about 30 us, a matrix 0.25 ns a byte)
+    double fill_us = 0.25e-3 * (double)host_bytes;
     for (const Block &b : plan) fill_us += b.kind == BK_PHASE ? 30 : 0;
+    unsigned char *hm = (unsigned char *)st->h_mats;
     parallel_blocks(plan.size(), fill_us, [&](size_t i) {
-      if (mat_off[i] != (size_t)-1 && !dev_operand_bytes(plan[i]))
-        fill_dev_matrix(plan[i], c128, (unsigned char *)st->h_mats + mat_off[i]);
+      if (host_off[i] != none) fill_dev_matrix(plan[i], c128, hm + host_off[i]);
     });
-    if (operand_bytes) fill_operand_program(plan, (unsigned char *)st->h_mats + prog_off);
-    e = cudaMemcpyAsync(st->d_mats, st->h_mats, mat_bytes, cudaMemcpyHostToDevice, st->stream);
+    if (tile_off < dev_bytes) fill_operand_program(plan, hm + prog_off);
+    if (up_bytes) e = cudaMemcpyAsync(dm, hm, up_bytes, cudaMemcpyHostToDevice, st->stream);
+    for (const Slots &x : slots)
+      if (e == cudaSuccess && x.count)
+        e = cudaMemcpy2DAsync(dm + x.dev, x.slot, hm + x.host, x.mat, x.mat, x.count, cudaMemcpyHostToDevice, st->stream);
     if (e != cudaSuccess) return cuda_fail(st, e, "qs_apply_circuit");
     e = cudaEventRecord(st->mats_copied, st->stream);
     if (e == cudaSuccess && any_tc) e = make_dev_operands(plan, mat_off, c128, st->d_mats, st->stream);
-    if (e == cudaSuccess && operand_bytes)
-      e = build_dev_operands((unsigned char *)st->d_mats + prog_off, (unsigned char *)st->d_mats + mat_bytes, operand_bytes,
-                             st->stream);
+    if (e == cudaSuccess && tile_off < dev_bytes)
+      e = build_dev_operands(dm + prog_off, dm + tile_off, dev_bytes - tile_off, st->stream);
     if (e != cudaSuccess) return cuda_fail(st, e, "qs_apply_circuit");
   }
 
@@ -448,7 +463,9 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
   st->recs.reserve(plan.size());
   st->h2d_bytes = 0;
   if (resident) {
-    e = run_resident(st->amps, st->n, plan, st->stream);
+    size_t sent = 0;
+    e = run_resident(st->amps, st->n, plan, st->stream, &sent);
+    st->h2d_bytes = (double)sent;
     if (e != cudaSuccess) return cuda_fail(st, e, "qs_apply_circuit launch");
   }
   for (size_t i = 0; i < plan.size(); i++) {
@@ -468,7 +485,7 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
     r.tiles = shape.tiles;
     r.ctas = shape.ctas;
     st->rec_class.push_back(block_class(b));
-    st->h2d_bytes += (double)block_param_bytes(b, c128);
+    if (!resident) st->h2d_bytes += (double)block_param_bytes(b, c128);
     st->recs.push_back(r);
   }
   std::memcpy(st->perm, perm, sizeof(perm));

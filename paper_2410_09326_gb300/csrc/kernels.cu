@@ -693,7 +693,7 @@ __global__ void __launch_bounds__(256) k_distance(const Ta *__restrict__ a, cons
 }
 
 template <typename T> size_t param_bytes_t(const Block &b) {
-  if (b.kind == BK_TILE && b.tc) return operand_program_bytes({b});
+  if (b.kind == BK_TILE && b.tc) return operand_program_bytes(&b, 1);
   if (b.kind == BK_TILE) return 2 * sizeof(T *) + sizeof(long long) + tile_desc_bytes(b, sizeof(T) == 16);
   if (b.kind == BK_PHASE) return 2 * sizeof(T *) + sizeof(long long) + phase_desc_bytes(b, sizeof(T) == 16);
   if (b.kind == BK_PERMUTE) return sizeof(T *) + sizeof(long long) + 2 * sizeof(int);

@@ -1,6 +1,6 @@
 // Operands of single tensor-core blocks, made on the device.
 //
-// A block's upload holds its matrix (FP32 for complex64, FP64 for complex128)
+// The upload leaves a block's matrix (FP32 for complex64, FP64 for complex128)
 // at the start of the space its B operand takes; one launch per call turns
 // every matrix into B in place: FP16 halves for tc16.cu and tc16x.cu, digit
 // planes for tc64.cu. The host made them before, two software FP16
@@ -92,9 +92,7 @@ __global__ void __launch_bounds__(256) k_operands(const __grid_constant__ Jobs p
 
 }  // namespace
 
-// Whether the block's operand is made here from its matrix.
-static bool job_of(const Block &b, bool c128, size_t at, Job &j) {
-  if (b.kind != BK_DENSE || !b.tc || b.tc_tf32) return false;
+static void job_of(const Block &b, bool c128, size_t at, Job &j) {
   j.at = (uint32_t)(at >> 8);
   j.c128 = c128;
   j.k = (uint8_t)b.k;
@@ -107,12 +105,13 @@ static bool job_of(const Block &b, bool c128, size_t at, Job &j) {
   TcXLayout x;
   if (b.tc_xg && tc_exchange_layout(64, b, x))
     for (int s = 0; s < b.k; s++) j.slot[s] = (uint8_t)x.slot_mat[s];
-  return true;
 }
 
 }  // namespace kern
 
 using namespace kern;
+
+bool made_on_device(const Block &b) { return b.kind == BK_DENSE && b.tc && !b.tc_tf32; }
 
 cudaError_t make_dev_operands(const std::vector<Block> &plan, const std::vector<size_t> &off, bool c128, void *base,
                               cudaStream_t s) {
@@ -121,7 +120,7 @@ cudaError_t make_dev_operands(const std::vector<Block> &plan, const std::vector<
   for (size_t i = 0; i < plan.size();) {
     int n = 0;
     for (; i < plan.size() && n < kJobs; i++)
-      if (off[i] != (size_t)-1 && job_of(plan[i], c128, off[i], p.job[n])) n++;
+      if (made_on_device(plan[i])) job_of(plan[i], c128, off[i], p.job[n++]);
     if (!n) continue;
     k_operands<<<n, 256, 0, s>>>(p);
     cudaError_t e = cudaGetLastError();

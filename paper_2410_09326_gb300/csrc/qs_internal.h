@@ -210,15 +210,17 @@ cudaError_t launch_block(void *amps, int n, bool c128, const Block &b, cudaStrea
 bool block_needs_dev_matrix(const Block &b, bool c128);
 size_t block_dev_matrix_bytes(const Block &b, bool c128);
 void fill_dev_matrix(const Block &b, bool c128, void *host_out);
-// Single tensor-core blocks: makes their operands on the device, in place, from
-// the matrices that fill_dev_matrix wrote at off[i] (-1: none) behind base.
+// Single tensor-core blocks: the device makes their operands
+// (block_dev_matrix_bytes), in place, from the matrices that fill_dev_matrix
+// wrote and an upload left at off[i] behind base.
+bool made_on_device(const Block &b);
 cudaError_t make_dev_operands(const std::vector<Block> &plan, const std::vector<size_t> &off, bool c128, void *base,
                               cudaStream_t s);
 // Tensor-core tile passes read operands that a launch makes on the device from
 // their members' gates: their size (0 for other blocks), and for all passes of
 // a plan, the gates as uploaded (program) and the launch.
 size_t dev_operand_bytes(const Block &b);
-size_t operand_program_bytes(const std::vector<Block> &plan);
+size_t operand_program_bytes(const Block *blocks, size_t count);
 void fill_operand_program(const std::vector<Block> &plan, void *out);
 cudaError_t build_dev_operands(const void *program, void *out, size_t bytes, cudaStream_t s);
 // Bytes of gate data one block ships to the device: its kernel parameters
@@ -230,10 +232,10 @@ cudaError_t launch_block_with_matrix(void *amps, int n, bool c128, const Block &
                                      int *err, cudaStream_t s, int threads, LaunchShape *shape = nullptr);
 // Narrow complex64 states (resident.cu): whether the whole plan can run in
 // shared memory, and the launches that do it (as few as its records fit the
-// kernel parameters).
+// kernel parameters; *sent receives their bytes).
 constexpr int kResidentBits = 13;
 bool resident_applies(const std::vector<Block> &plan, int n);
-cudaError_t run_resident(void *amps, int n, const std::vector<Block> &plan, cudaStream_t s);
+cudaError_t run_resident(void *amps, int n, const std::vector<Block> &plan, cudaStream_t s, size_t *sent);
 cudaError_t launch_permute(void *amps, int n, bool c128, int a, int b, cudaStream_t s);
 // Disjoint exchanges of physical bits, all at once.
 cudaError_t launch_bit_swaps(void *amps, int n, bool c128, const std::vector<std::pair<int, int>> &swaps,

@@ -138,7 +138,7 @@ bool resident_applies(const std::vector<Block> &plan, int n) {
   return true;
 }
 
-cudaError_t run_resident(void *amps, int n, const std::vector<Block> &plan, cudaStream_t s) {
+cudaError_t run_resident(void *amps, int n, const std::vector<Block> &plan, cudaStream_t s, size_t *sent) {
   // a thread per group of eight amplitudes, no fewer than two warps
   const int threads = n >= 13 ? 1024 : (n <= 9 ? 64 : 1 << (n - 3));
   const size_t smem_max = (sizeof(float2) << kResidentBits) + sizeof(uint4) * kProgWords;
@@ -169,6 +169,7 @@ cudaError_t run_resident(void *amps, int n, const std::vector<Block> &plan, cuda
     else k_resident<512><<<1, threads, smem, s>>>(p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    *sent += sizeof(p);
   }
   return cudaSuccess;
 }

@@ -630,9 +630,10 @@ cudaError_t run_tc_tile(float2 *a, int n, const Block &b, const void *dev_b, int
 
 using namespace kern;
 
-size_t operand_program_bytes(const std::vector<Block> &plan) {
+size_t operand_program_bytes(const Block *blocks, size_t count) {
   size_t products = 0, words = 0;
-  for (const Block &b : plan) {
+  for (size_t i = 0; i < count; i++) {
+    const Block &b = blocks[i];
     if (!dev_operand_bytes(b)) continue;
     products += tc_tile_mats(b);
     for (const Block &m : b.sub) words += 1 + m.gates.size() + m.mat.size();

@@ -79,3 +79,21 @@ def test_batch_of_wide_circuits():
         finally:
             for st in states:
                 qs.qs_free_state(st)
+
+
+def test_bytes_shipped_are_those_of_the_launches():
+    """A narrow state's gate data are its records, in the parameters of its launches."""
+    n = 12
+    st = qs.qs_alloc_state(n, qs.QS_C64)
+    try:
+        shipped = []
+        for layers in (2, 40):
+            gates = qs.gates_to_array(cg.random_layered(n, layers, cg.SplitMix64(layers)))
+            qs.qs_apply_circuit(st, gates, qs.QS_PGO_RULES)
+            summary, recs = qs.qs_profile(st)
+            assert len(recs) > 1 and all(r.tiles == 0 for r in recs)
+            shipped.append(summary.h2d_bytes)
+        # launch parameters of 32 KB, whole; the matrices of the deeper circuit's blocks take several
+        assert 32000 < shipped[0] < 32764 and shipped[1] % shipped[0] == 0 and shipped[1] > shipped[0]
+    finally:
+        qs.qs_free_state(st)
