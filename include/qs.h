@@ -87,7 +87,8 @@ typedef struct {
 #define QS_VSWAP ((uint64_t)1 << 0)         /* SWAPs become relabellings of perm */
 #define QS_FUSE ((uint64_t)1 << 1)          /* k-qubit fusion, k from QS_FUSE_K */
 #define QS_DIAG ((uint64_t)1 << 2)          /* diagonal runs fuse, any width */
-#define QS_TC ((uint64_t)1 << 3)            /* dense k>=4 blocks on tensor cores (opts->tc_precision) */
+#define QS_TC ((uint64_t)1 << 3)            /* dense blocks on the tensor cores: complex64 4..6 targets,
+                                               complex128 4 and 5 (opts->tc_precision) */
 #define QS_PROFILE ((uint64_t)1 << 4)       /* time every block with CUDA events */
 #define QS_RELOCATE ((uint64_t)1 << 5)      /* profile-guided hot-qubit relocation */
 #define QS_FOLD ((uint64_t)1 << 6)          /* rotation folding + pair cancellation first */
@@ -108,7 +109,14 @@ typedef struct {
   int diag_max;         /* widest diagonal phase table, 1..QS_MAX_DIAG (wider runs: polynomials) */
   int threads;          /* launch override: threads per CTA (0 = tuned default) */
   double peak_gbs;      /* HBM copy bandwidth the cost model scales its priors by */
-  int tc_precision;     /* QS_TC operands: 0 = two FP16 halves (k = 4..6), 1 = 3 x TF32 (k = 4, 5) */
+  int tc_precision;     /* QS_TC operands, complex64: 0 = two FP16 halves (k = 4..6), 1 = 3 x TF32
+                           (k = 4, 5). complex128: 0 = exact digit planes (k = 4, 5) with one
+                           rounding of the result: a block's error is below 1e-16 of its group of
+                           2^k amplitudes (the FP64 kernel's 3e-16), 2^-54 of the group's largest in
+                           any of them; groups in which an amplitude lies below 2^-20 of the
+                           largest, where the matrix may keep the two apart, take FP64 arithmetic,
+                           so that small amplitudes keep their own precision; 1 = the FP64 kernel
+                           for every group. QS_PGO_RULES chooses QS_TC for both types */
   int test_wait_timeout; /* test hook, 0 in normal use: tensor-core blocks withhold their
                             completion signal, so their bounded (1 s) wait runs out and the
                             next synchronising call returns QS_ETIMEOUT; results invalid */

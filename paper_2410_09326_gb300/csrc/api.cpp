@@ -364,45 +364,62 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
                         resident_applies(plan, st->n);
   // Device data: matrices, tables and the gates of tile passes as they are
   // staged; then the operands of single tensor-core blocks, of which the
-  // matrices alone are staged (an eighth to a half of the operand) and spread
+  // matrices alone are staged (a quarter or half of the operand) and spread
   // over equal slots, k by k; then the operands of tile passes.
   const size_t none = (size_t)-1;
-  std::vector<size_t> mat_off(plan.size(), none), host_off(plan.size(), none);
-  size_t up_bytes = 0;
-  for (size_t i = 0; i < plan.size(); i++)
-    if (!resident && block_needs_dev_matrix(plan[i], c128) && !made_on_device(plan[i])) {
-      mat_off[i] = host_off[i] = up_bytes;
-      up_bytes += (block_dev_matrix_bytes(plan[i], c128) + 255) & ~(size_t)255;
-    }
-  const size_t prog_off = up_bytes;
-  if (tiles) up_bytes += (operand_program_bytes(plan.data(), plan.size()) + 255) & ~(size_t)255;
+  std::vector<size_t> mat_off, host_off;
   struct Slots {
     size_t dev, host, slot, mat, count;
+    size_t at;  // of the matrix in its slot
   } slots[3];
-  size_t dev_bytes = up_bytes, host_bytes = up_bytes;
-  for (int k = 4; k <= 6; k++) {
-    Slots &x = slots[k - 4];
-    x = {dev_bytes, host_bytes, 0, 0, 0};
-    for (size_t i = 0; i < plan.size(); i++) {
-      if (resident || !made_on_device(plan[i]) || plan[i].k != k) continue;
-      x.slot = (block_dev_matrix_bytes(plan[i], c128) + 255) & ~(size_t)255;
-      x.mat = plan[i].mat.size() * (c128 ? 16 : 8);
-      mat_off[i] = x.dev + x.count * x.slot;
-      host_off[i] = x.host + x.count * x.mat;
-      x.count++;
+  size_t up_bytes, prog_off, tile_off, dev_bytes, host_bytes;
+  auto lay_out = [&] {
+    mat_off.assign(plan.size(), none);
+    host_off.assign(plan.size(), none);
+    up_bytes = 0;
+    for (size_t i = 0; i < plan.size(); i++)
+      if (!resident && block_needs_dev_matrix(plan[i], c128) && !made_on_device(plan[i])) {
+        mat_off[i] = host_off[i] = up_bytes;
+        up_bytes += (block_dev_matrix_bytes(plan[i], c128) + 255) & ~(size_t)255;
+      }
+    prog_off = up_bytes;
+    if (tiles) up_bytes += (operand_program_bytes(plan.data(), plan.size()) + 255) & ~(size_t)255;
+    dev_bytes = host_bytes = up_bytes;
+    for (int k = 4; k <= 6; k++) {
+      Slots &x = slots[k - 4];
+      x = {dev_bytes, host_bytes, 0, 0, 0, 0};
+      for (size_t i = 0; i < plan.size(); i++) {
+        if (resident || !made_on_device(plan[i]) || plan[i].k != k) continue;
+        x.slot = (block_dev_matrix_bytes(plan[i], c128) + 255) & ~(size_t)255;
+        x.mat = plan[i].mat.size() * (c128 ? 16 : 8);
+        x.at = dev_matrix_at(plan[i], c128);
+        mat_off[i] = x.dev + x.count * x.slot;
+        host_off[i] = x.host + x.count * x.mat;
+        x.count++;
+      }
+      dev_bytes += x.count * x.slot;
+      host_bytes += x.count * x.mat;
     }
-    dev_bytes += x.count * x.slot;
-    host_bytes += x.count * x.mat;
+    tile_off = dev_bytes;
+    for (size_t i = 0; i < plan.size(); i++)
+      if (const size_t ob = dev_operand_bytes(plan[i])) {
+        mat_off[i] = dev_bytes;
+        dev_bytes += ob;
+      }
+  };
+  lay_out();
+  unsigned char *dm = (unsigned char *)st->d_mats;
+  cudaError_t e = grow(dm, st->mats_cap, dev_bytes);
+  if (e != cudaSuccess && c128) {
+    // digit planes take five times the matrices' memory: without it, the FP64 kernels
+    for (Block &b : plan) b.tc = false;
+    lay_out();
+    e = grow(dm, st->mats_cap, dev_bytes);
   }
-  const size_t tile_off = dev_bytes;
-  for (size_t i = 0; i < plan.size(); i++)
-    if (const size_t ob = dev_operand_bytes(plan[i])) {
-      mat_off[i] = dev_bytes;
-      dev_bytes += ob;
-    }
+  st->d_mats = dm;
+  if (e != cudaSuccess) return fail(QS_ENOMEM, "matrix buffer allocation failed");
   bool any_tc = false;
   for (const Block &b : plan) any_tc |= b.tc;
-  cudaError_t e;
   if (host_bytes) {
     if (st->mats_copied) {
       e = cudaEventSynchronize(st->mats_copied);  // staging buffer free again
@@ -419,10 +436,6 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
       if (e != cudaSuccess) return fail(QS_ENOMEM, "pinned staging allocation failed");
       st->h_mats_cap = host_bytes;
     }
-    unsigned char *dm = (unsigned char *)st->d_mats;
-    e = grow(dm, st->mats_cap, dev_bytes);
-    st->d_mats = dm;
-    if (e != cudaSuccess) return fail(QS_ENOMEM, "matrix buffer allocation failed");
     // (a phase polynomial's table takes about 30 us, a matrix 0.25 ns a byte)
     double fill_us = 0.25e-3 * (double)host_bytes;
     for (const Block &b : plan) fill_us += b.kind == BK_PHASE ? 30 : 0;
@@ -434,7 +447,7 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
     if (up_bytes) e = cudaMemcpyAsync(dm, hm, up_bytes, cudaMemcpyHostToDevice, st->stream);
     for (const Slots &x : slots)
       if (e == cudaSuccess && x.count)
-        e = cudaMemcpy2DAsync(dm + x.dev, x.slot, hm + x.host, x.mat, x.mat, x.count, cudaMemcpyHostToDevice, st->stream);
+        e = cudaMemcpy2DAsync(dm + x.dev + x.at, x.slot, hm + x.host, x.mat, x.mat, x.count, cudaMemcpyHostToDevice, st->stream);
     if (e != cudaSuccess) return cuda_fail(st, e, "qs_apply_circuit");
     e = cudaEventRecord(st->mats_copied, st->stream);
     if (e == cudaSuccess && any_tc) e = make_dev_operands(plan, mat_off, c128, st->d_mats, st->stream);

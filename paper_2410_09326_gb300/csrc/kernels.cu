@@ -443,7 +443,7 @@ size_t block_dev_matrix_bytes(const Block &b, bool c128) {
   if (!block_needs_dev_matrix(b, c128)) return 0;
   if (b.kind == BK_TILE) return tile_desc_bytes(b, c128);
   if (b.kind == BK_PHASE) return phase_desc_bytes(b, c128);
-  if (b.tc && c128) return tc64_b_bytes(b.k);
+  if (b.tc && c128) return tc64_b_bytes(b.k) + b.mat.size() * 16;  // the digits, then the matrix
   if (b.tc) return b.tc_tf32 ? tc_b_floats(b.k) * sizeof(float) : tc16_b_bytes(b.k);
   return b.mat.size() * (c128 ? 16 : 8);
 }

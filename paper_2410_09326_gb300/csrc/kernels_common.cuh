@@ -222,7 +222,8 @@ cudaError_t run_tc_tile(float2 *a, int n, const Block &b, const void *dev_b, int
                         LaunchShape *shape);
 
 // complex128 blocks on the tensor cores (tc64.cu), k = 4, 5: dev_b holds
-// tc64_b_bytes(k) bytes made by make_dev_operands: digit planes in that layout.
+// tc64_b_bytes(k) bytes made by make_dev_operands (digit planes in that layout)
+// and behind them the matrix they are made from.
 size_t tc64_b_bytes(int k);
 cudaError_t run_dense_tc64(double2 *a, int n, const Block &b, const void *dev_b, int *err, cudaStream_t s,
                            LaunchShape *shape);

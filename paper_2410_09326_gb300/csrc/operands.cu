@@ -1,13 +1,13 @@
 // Operands of single tensor-core blocks, made on the device.
 //
 // The upload leaves a block's matrix (FP32 for complex64, FP64 for complex128)
-// at the start of the space its B operand takes; one launch per call turns
-// every matrix into B in place: FP16 halves for tc16.cu and tc16x.cu, digit
-// planes for tc64.cu. The host made them before, two software FP16
+// at the start of the space its B operand takes, or behind it where tc64.cu
+// needs the matrix too; one launch per call turns every matrix into B: FP16
+// halves for tc16.cu and tc16x.cu, digit planes for tc64.cu. The host made them before, two software FP16
 // conversions per entry and half: 50 us a 5-target block, 230 us one of 6,
 // 105 us a complex128 one, spread over the host's threads while the GPU
 // waited. One CTA per block: it reads the matrix into shared memory, then
-// writes B over it. The complex128 digits are bound by the FP64 rate (80
+// writes B (over it, for complex64). The complex128 digits are bound by the FP64 rate (80
 // operations an entry at two per clock).
 #include <cstring>
 
@@ -24,6 +24,7 @@ constexpr int kSrcBytes = 32 * 1024;  // 64 x 64 complex64, the largest matrix
 
 struct Job {
   uint32_t at;     // of the block's operand, in 256 bytes
+  uint16_t src;    // of its matrix behind that, in 256 bytes
   uint8_t c128, k;
   uint8_t slot[6]; // slot bit -> target's position (complex64)
 };
@@ -39,10 +40,11 @@ __global__ void __launch_bounds__(256) k_operands(const __grid_constant__ Jobs p
   __shared__ uint8_t pi[64];  // row or column of the matrix for one of B
   const Job j = p.job[blockIdx.x];
   unsigned char *op = p.base + ((size_t)j.at << 8);
+  const unsigned char *in = op + ((size_t)j.src << 8);
   const int D = 1 << j.k, KR = 2 * D;
   const int words = (D * D * (j.c128 ? 16 : 8)) / 16;
   for (int i = threadIdx.x; i < words; i += 256)
-    reinterpret_cast<uint4 *>(src)[i] = reinterpret_cast<const uint4 *>(op)[i];
+    reinterpret_cast<uint4 *>(src)[i] = reinterpret_cast<const uint4 *>(in)[i];
   if (threadIdx.x < D) {
     int s = 0;
     for (int b = 0; b < j.k; b++)
@@ -94,6 +96,7 @@ __global__ void __launch_bounds__(256) k_operands(const __grid_constant__ Jobs p
 
 static void job_of(const Block &b, bool c128, size_t at, Job &j) {
   j.at = (uint32_t)(at >> 8);
+  j.src = (uint16_t)(dev_matrix_at(b, c128) >> 8);
   j.c128 = c128;
   j.k = (uint8_t)b.k;
   for (int s = 0; s < 6; s++) j.slot[s] = (uint8_t)s;
@@ -110,6 +113,8 @@ static void job_of(const Block &b, bool c128, size_t at, Job &j) {
 }  // namespace kern
 
 using namespace kern;
+
+size_t dev_matrix_at(const Block &b, bool c128) { return c128 ? tc64_b_bytes(b.k) : 0; }
 
 bool made_on_device(const Block &b) { return b.kind == BK_DENSE && b.tc && !b.tc_tf32; }
 

@@ -982,6 +982,16 @@ qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<
   return QS_OK;
 }
 
+int digit_check(const std::vector<cd> &m) {
+  const double least = std::ldexp(1.0, -2 * kDigitSpan);
+  int check = 0;
+  for (const cd &z : m) {
+    const double s = std::norm(z);
+    if (s < least) check = std::max(check, z == cd(0, 0) ? 1 : 2);
+  }
+  return check;
+}
+
 }  // namespace
 
 void parallel_blocks(size_t n, double work_us, const std::function<void(size_t)> &f) { parallel_for(n, work_us, f); }
@@ -1243,9 +1253,11 @@ qs_status build_plan(int n, const qs_gate *gates, size_t n_gates, uint64_t flags
       b.tc_max_ctas = opts.tc_max_ctas;
       continue;
     }
-    // complex128 blocks run on FP16 digit planes (tc64.cu), 4 and 5 targets
-    b.tc = (flags & QS_TC) && b.kind == BK_DENSE && b.k >= 4 && b.k <= (tf32 || c128 ? 5 : 6);
-    b.tc_tf32 = b.tc && tf32 && !c128;
+    // complex128 blocks run on FP16 digit planes (tc64.cu), 4 and 5 targets,
+    // or keep the FP64 kernel where the options ask for the other precision
+    b.tc = (flags & QS_TC) && b.kind == BK_DENSE && b.k >= 4 && b.k <= (tf32 || c128 ? 5 : 6) && !(c128 && tf32);
+    if (b.tc && c128) b.digit_check = digit_check(b.mat);
+    b.tc_tf32 = b.tc && tf32;
     b.shuffles = opts.no_shuffles == 0;
     // lane-exchange gathers where they measured faster (tc_exchange_pays),
     // or everywhere the layout allows with tc_exchange = 2

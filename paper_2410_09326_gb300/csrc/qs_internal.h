@@ -48,6 +48,7 @@ enum BlockKind : uint8_t { BK_DENSE = 0, BK_DIAG = 1, BK_PERMUTE = 2, BK_TILE = 
 constexpr int kMaxFixed = 24;  // targets + controls handled by the index insert
 constexpr int kMaxTileBits = 14;  // widest shared-memory tile (QS_TILE)
 constexpr int kTileLowBits = 4;   // contiguous low bits every tile includes (128-byte c64 runs)
+constexpr int kDigitSpan = 20;    // complex128 digit planes (tc64.cu): powers of two between a group's amplitudes
 constexpr int kTcTileBits = 12;       // tile of a tensor-core pass (tc_tile.cu): 32 KiB
 constexpr int kTcTileMaxBlocks = 32;  // its blocks in one launch
 constexpr int kTcTileSel = 2;         // bits outside the tile that pick a block's matrix
@@ -66,6 +67,11 @@ struct Block {
   bool tc_tf32 = false;           // tensor-core operands: 3 x TF32 instead of 2 x FP16
   bool shuffles = true;           // CUDA-core blocks with low targets: warp-shuffle kernel
   bool tc_xg = false;             // 4..6-target tensor-core blocks: lane-exchange gathers (tc16x.cu)
+  // complex128 tensor-core blocks: which groups must be looked at for small
+  // amplitudes (tc64.cu). 0: none, the matrix mixes every amplitude into every
+  // result with a weight of 2^-kDigitSpan at least; 1: it has zeros; 2: and
+  // nonzero entries below that
+  int digit_check = 0;
   bool withhold_commit = false;   // test hook (qs_opts.test_wait_timeout)
   int tc_max_ctas = 0;            // test hook (qs_opts.tc_max_ctas): cap on tensor-core and phase CTAs
   // tile pass (BK_TILE): k = tile qubits, tile_q their physical positions
@@ -210,10 +216,11 @@ cudaError_t launch_block(void *amps, int n, bool c128, const Block &b, cudaStrea
 bool block_needs_dev_matrix(const Block &b, bool c128);
 size_t block_dev_matrix_bytes(const Block &b, bool c128);
 void fill_dev_matrix(const Block &b, bool c128, void *host_out);
-// Single tensor-core blocks: the device makes their operands
-// (block_dev_matrix_bytes), in place, from the matrices that fill_dev_matrix
-// wrote and an upload left at off[i] behind base.
+// Single tensor-core blocks: the device makes their operands (at off[i] behind
+// base, block_dev_matrix_bytes) from the matrices that fill_dev_matrix wrote and
+// an upload left dev_matrix_at behind their start: in place for complex64.
 bool made_on_device(const Block &b);
+size_t dev_matrix_at(const Block &b, bool c128);
 cudaError_t make_dev_operands(const std::vector<Block> &plan, const std::vector<size_t> &off, bool c128, void *base,
                               cudaStream_t s);
 // Tensor-core tile passes read operands that a launch makes on the device from

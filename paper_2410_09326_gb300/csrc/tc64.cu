@@ -29,6 +29,18 @@
 // with amplitudes spread over 2^60 by 1.0e-16 to 1.5e-16 against 1.8e-16 to
 // 2.8e-16.
 //
+// The digits keep 54 bits of a group's largest amplitude, and as much less of a
+// small one as it is smaller. FP64 sums lose that too where the matrix mixes
+// the large amplitude into every result, but keep small amplitudes' own 53
+// bits where it holds them apart (zeros of the matrix) or brings little over
+// (small entries). So groups are looked at where the matrix has entries below
+// 2^-16: if an amplitude lies below 2^-16 of the largest (zeros count where
+// small entries are not zero), the group takes the FP64 mat-vec (exact_groups).
+// On random circuits that costs 1% (10 layers, 24 qubits, 8.69 -> 8.78 ms;
+// most of it the look), in early layers up to an FP64 pass for a block (one of
+// ten 4-layer circuits 4.2 -> 5.9 ms). At 2^-12 three in ten took 1.1 to 2.2
+// times as long, at 2^-20 none.
+//
 // Measured at n = 25 (1 GiB read and written), FP64 kernel -> this one: 5
 // targets 6930 -> 430 us, 4 targets 4080 -> 330 us (3.2 TB/s); bits 0..4:
 // 499 us, bits 0..3: 403 us. What bounds it is issue and latency: about 75
@@ -137,9 +149,37 @@ __device__ __noinline__ double scale_back_slow(long long v, int gexp) {
   return scalbn(__ll2double_rn(v), gexp - 1081);
 }
 
+// The tile's groups that `rows` marks, by the FP64 mat-vec, a warp a group and
+// a lane a result. Their amplitudes are still the block's input.
+template <int K>
+__device__ __noinline__ void exact_groups(double2 *a, const double2 *mat, const TcParam &p, long long tile,
+                                          const uint32_t *rows) {
+  constexpr int D = 1 << K;
+  const int lane = threadIdx.x & 31, r = lane & (D - 1);
+  uint64_t off = 0;
+#pragma unroll
+  for (int j = 0; j < K; j++)
+    if ((r >> j) & 1) off += 1ull << p.tq[j];
+  for (int row = threadIdx.x >> 5; row < 128; row += Tc64<K>::NT / 32) {
+    if (!((rows[row >> 5] >> (row & 31)) & 1)) continue;  // the same for the whole warp
+    double2 *x = a + ((insert_zeros((uint64_t)(tile * 128 + row), p.fixed, p.nf) | p.cmask) + off);
+    const double2 v = *x;
+    double re = 0, im = 0;
+    for (int c = 0; c < D; c++) {
+      const double2 w = mat[r * D + c];
+      const double vx = __shfl_sync(0xffffffffu, v.x, c), vy = __shfl_sync(0xffffffffu, v.y, c);
+      re = fma(w.x, vx, re);
+      re = fma(-w.y, vy, re);
+      im = fma(w.x, vy, im);
+      im = fma(w.y, vx, im);
+    }
+    if (lane < D) *x = make_double2(re, im);
+  }
+}
+
 template <int K>
 __global__ void __launch_bounds__(Tc64<K>::NT, Tc64<K>::CTAS)
-    k_dense_tc64(double2 *__restrict__ a, const uint4 *__restrict__ bmat, const __grid_constant__ TcParam p,
+    k_dense_tc64(double2 *__restrict__ a, const uint4 *__restrict__ bmat, const __grid_constant__ TcParam p, int check,
                  int *__restrict__ err) {
   using C = Tc64<K>;
   constexpr int KR = C::KR, NT = C::NT;
@@ -149,7 +189,8 @@ __global__ void __launch_bounds__(Tc64<K>::NT, Tc64<K>::CTAS)
   unsigned char *sB = smem + kDigitsA * C::A_BYTES;
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ uint32_t tmem_slot;
-  __shared__ uint32_t red[NT];
+  __shared__ uint32_t red[2][NT];
+  __shared__ uint32_t exact_rows[4];
 
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
@@ -205,18 +246,25 @@ __global__ void __launch_bounds__(Tc64<K>::NT, Tc64<K>::CTAS)
   gather(tile);
 
   for (; tile < p.n_tiles; tile += gridDim.x) {
-    // the group's exponent: the largest high word without its sign
-    uint32_t mx = 0;
+    // the group's exponent: the largest high word without its sign; and that
+    // of its smallest amplitude (check 1: of the nonzero ones)
+    uint32_t mx = 0, mn = 0x7fffffffu;
 #pragma unroll
     for (int u = 0; u < 8; u++) {
-      mx = max(mx, (uint32_t)__double2hiint(v[u].x) & 0x7fffffffu);
-      mx = max(mx, (uint32_t)__double2hiint(v[u].y) & 0x7fffffffu);
+      const uint32_t m = max((uint32_t)__double2hiint(v[u].x) & 0x7fffffffu, (uint32_t)__double2hiint(v[u].y) & 0x7fffffffu);
+      mx = max(mx, m);
+      mn = min(mn, check == 1 && m == 0 ? 0x7fffffffu : m);
     }
-    red[tid] = mx;
+    red[0][tid] = mx;
+    if (check) red[1][tid] = mn;
     if (!__syncthreads_and(ok)) break;  // a wait of the last tile ran out
 #pragma unroll
-    for (int o = 1; o < C::TPR; o++) mx = max(mx, red[(tid + o * 128) % NT]);
+    for (int o = 1; o < C::TPR; o++) {
+      mx = max(mx, red[0][(tid + o * 128) % NT]);
+      if (check) mn = min(mn, red[1][(tid + o * 128) % NT]);
+    }
     const int gexp = max((int)(mx >> 20), 1);  // subnormals count from exponent 1
+    const bool exact = check && gexp < 2047 && gexp - (int)(mn >> 20) > kDigitSpan;
 #pragma unroll
     for (int hh = 0; hh < 2; hh++) {
       uint64_t f[8];
@@ -283,13 +331,19 @@ __global__ void __launch_bounds__(Tc64<K>::NT, Tc64<K>::CTAS)
           if (!normal && fx != 0) y[i] = scale_back_slow(fx, gexp);
           if (not_finite) y[i] = __hiloint2double(0x7ff80000, 0);
         }
-        if (cur_valid) {
+        if (cur_valid && !exact) {
           cur[offset(4 * hh + 2 * c)] = make_double2(y[0], y[1]);
           cur[offset(4 * hh + 2 * c + 1)] = make_double2(y[2], y[3]);
         }
       }
     }
     phase ^= 1;
+    if (check && __syncthreads_or(exact)) {
+      const uint32_t rows = __ballot_sync(0xffffffffu, exact);
+      if (tid < 128 && (tid & 31) == 0) exact_rows[warp] = rows;
+      __syncthreads();
+      exact_groups<K>(a, reinterpret_cast<const double2 *>(bmat + C::B_BYTES / 16), p, tile, exact_rows);
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   if (!__syncthreads_and(ok)) {
@@ -332,7 +386,7 @@ cudaError_t run_tc64(double2 *a, int n, const Block &b, const void *dev_b, int *
     shape->tiles = p.n_tiles;
     shape->ctas = grid;
   }
-  k_dense_tc64<K><<<grid, Tc64<K>::NT, Tc64<K>::SMEM, s>>>(a, (const uint4 *)dev_b, p, err);
+  k_dense_tc64<K><<<grid, Tc64<K>::NT, Tc64<K>::SMEM, s>>>(a, (const uint4 *)dev_b, p, b.digit_check, err);
   return cudaGetLastError();
 }
 

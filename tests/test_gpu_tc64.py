@@ -132,3 +132,80 @@ def test_timeout_is_reported(k):
         assert abs(qs.qs_norm(st) - 1) < 1e-14
     finally:
         qs.qs_free_state(st)
+
+
+# explicit flags, and the rules (which take blocks of five targets)
+@pytest.mark.parametrize("flags", [qs.QS_FUSE | qs.QS_FUSE_K(5) | qs.QS_TC, qs.QS_FUSE | qs.QS_FUSE_K(4) | qs.QS_TC,
+                                   qs.QS_PGO_RULES])
+def test_small_rotations_keep_their_small_amplitudes(flags):
+    """RX(2e-9) on every qubit of |0...0>: an amplitude with j flips is 1e-9 to the j, each exact to FP64."""
+    n, t = 10, 2e-9
+    st = qs.qs_alloc_state(n, qs.QS_C128)
+    try:
+        qs.qs_apply_circuit(st, qs.gates_to_array([("rx", [q], [t]) for q in range(n)]), flags)
+        assert sum(r.tc for r in qs.qs_profile(st)[1]) >= 2
+        got = qs.qs_read_state(st, n, qs.QS_C128, logical_order=True)
+    finally:
+        qs.qs_free_state(st)
+    flips = np.array([bin(i).count("1") for i in range(1 << n)])
+    want = (-1j) ** flips * np.sin(t / 2) ** flips * np.cos(t / 2) ** (n - flips)
+    # two to three blocks of FP64 products of gates and amplitudes, 2^6 roundings each at most
+    assert (np.abs(got - want) <= 3 * 2.0 ** (6 - 53) * np.abs(want)).all()
+
+
+@pytest.mark.parametrize("targets", [[0, 1, 2, 3], [0, 1, 2, 3, 4], [1, 4, 6, 9], [2, 3, 7, 8, 11]])
+@pytest.mark.parametrize("tiny", [0.0, 1e-7])
+def test_groups_of_very_different_amplitudes_take_fp64(targets, tiny):
+    """A matrix that mixes one qubit and moves the others about keeps small amplitudes apart from large ones."""
+    n, k, r = 12, len(targets), random.Random(len(targets))
+    gates = [("u3", [targets[0]], [1.1, 0.3, 0.7])]
+    gates += [("cx", [a, b], []) for _ in range(2) for a, b in zip(targets, targets[1:] + targets[:1])]
+    if tiny:  # weights far below 1 between the halves of another qubit
+        gates += [("ry", [targets[1]], [tiny])]
+    gates = qs.gates_to_array(gates)
+    rng = np.random.default_rng(3)
+    groups = 1 << (n - k)
+    y = (rng.standard_normal((groups, 1 << k)) + 1j * rng.standard_normal((groups, 1 << k)))
+    wide = rng.random(groups) < 0.5   # groups that span 2^60; in the others no two amplitudes are more than 2 apart
+    y /= np.abs(y)
+    y[wide] *= np.exp2(rng.integers(-60, 0, (wide.sum(), 1 << k)))
+    y[~wide] *= 1 + rng.random(((~wide).sum(), 1 << k))
+    if not tiny:
+        y[rng.random(y.shape) < 0.1] = 0  # exact zeros stay out of it
+    y[7] = 0
+    idx = np.arange(1 << n)
+    low = idx[(idx & sum(1 << q for q in targets)) == 0]
+    at = low[:, None] + np.array([sum(((s >> j) & 1) << q for j, q in enumerate(targets)) for s in range(1 << k)])
+    x = np.zeros(1 << n, dtype=np.complex128)
+    x[at] = y
+    got, recs, width = _run(n, gates, x)
+    assert [(q.k, q.tc) for q in recs] == [(k, 1)]
+    _, (mat,), _ = qs.qs_plan(n, gates, qs.QS_FUSE | qs.QS_FUSE_K(width))
+    m = mat.astype(np.clongdouble)
+    want = np.stack([(m * v).sum(1) for v in y.astype(np.clongdouble)])
+    size = np.abs(y) @ np.abs(mat).T  # what an FP64 sum's error is relative to
+    err = np.abs(got[at] - want).astype(np.float64)
+    assert (err[wide] <= 2.0 ** (k + 1 - 53) * size[wide]).all()
+    # digits: 2^-54 of the largest amplitude for each of the inputs of a result, and its rounding
+    assert (err[~wide] <= (2.0 ** (k / 2 - 54) + 2.0 ** -53) * np.abs(y[~wide]).max(1, initial=0)[:, None] * 2).all()
+    assert (got[at][7] == 0).all()
+
+
+def test_the_other_precision_and_scarce_memory_take_the_fp64_kernel():
+    n = 14
+    gates = _gates([0, 2, 5, 9, 13], None, 8)
+    rng = np.random.default_rng(4)
+    x = rng.standard_normal(1 << n) + 1j * rng.standard_normal(1 << n)
+    opts = qs.qs_default_opts()
+    opts.tc_precision = 1
+    want, recs, _ = _run(n, gates, x, opts)
+    assert [r.tc for r in recs] == [0]
+    digits, recs, _ = _run(n, gates, x)
+    assert [r.tc for r in recs] == [1]
+    qs.qs_set_memory_limit(qs.qs_memory_in_use() + 40 * 1024)  # the matrix (16 KB), not its digits
+    try:
+        got, recs, _ = _run(n, gates, x)
+    finally:
+        qs.qs_set_memory_limit(0)
+    assert [r.tc for r in recs] == [0] and np.array_equal(got, want)
+    assert np.linalg.norm(digits - want) <= 4e-16 * np.linalg.norm(want)
