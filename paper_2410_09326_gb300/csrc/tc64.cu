@@ -34,12 +34,12 @@
 // the large amplitude into every result, but keep small amplitudes' own 53
 // bits where it holds them apart (zeros of the matrix) or brings little over
 // (small entries). So groups are looked at where the matrix has entries below
-// 2^-16: if an amplitude lies below 2^-16 of the largest (zeros count where
+// 2^-20: if an amplitude lies below 2^-20 of the largest (zeros count where
 // small entries are not zero), the group takes the FP64 mat-vec (exact_groups).
-// On random circuits that costs 1% (10 layers, 24 qubits, 8.69 -> 8.78 ms;
-// most of it the look), in early layers up to an FP64 pass for a block (one of
-// ten 4-layer circuits 4.2 -> 5.9 ms). At 2^-12 three in ten took 1.1 to 2.2
-// times as long, at 2^-20 none.
+// The look costs 3% (24 qubits, 10 layers, median of 60 random circuits 8.39 ->
+// 8.61 ms); a block whose groups all span more, as early layers with an angle
+// near a multiple of pi leave them, costs an FP64 pass: 3 of the 60 took 1.25
+// to 1.9 times as long (7 with 2^-16), the mean 8.43 -> 8.85 ms.
 //
 // Measured at n = 25 (1 GiB read and written), FP64 kernel -> this one: 5
 // targets 6930 -> 430 us, 4 targets 4080 -> 330 us (3.2 TB/s); bits 0..4:
