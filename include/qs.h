@@ -237,7 +237,8 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
 typedef struct {
   int32_t index;     /* launch order within the last apply call */
   uint8_t kind;      /* 0 dense block, 1 diagonal block, 2 physical bit exchange,
-                        3 tile pass (QS_TILE: several blocks in one HBM pass),
+                        3 tile pass (QS_TILE, or with tc = 1 tensor-core tile passes of the rules:
+                          several blocks in one HBM pass),
                         4 phase polynomial (a diagonal run wider than opts->diag_max),
                         5 exchange of a local bit (qubits[0]) with a global one (qubits[1])
                           (qs_plan with opts->n_global > 0) */
@@ -330,8 +331,9 @@ qs_status qs_pgo_predict(int n, qs_dtype dtype, const qs_gate *gates, size_t n_g
 
 /*
  * The host passes alone (virtual swap, fusion, classification), without a
- * GPU: the plan qs_apply_circuit would launch for a state of n qubits whose
- * map is *perm_inout (n entries, updated for absorbed SWAPs). Fills up to cap
+ * GPU: the plan qs_apply_circuit would launch for a complex64 state of n
+ * qubits (QS_PGO_RULES takes other block widths for narrow complex128 states,
+ * and no tensor-core tile passes for complex128) whose map is *perm_inout (n entries, updated for absorbed SWAPs). Fills up to cap
  * records (ms = -1) and, when mats is not NULL, the blocks' matrices in FP64
  * as interleaved (re, im) pairs, block after block: (2^k)^2 entries for a
  * dense block (row-major over the block's ascending physical qubits, local
@@ -340,7 +342,9 @@ qs_status qs_pgo_predict(int n, qs_dtype dtype, const qs_gate *gates, size_t n_g
  * (physical qubit, linear angle) pairs, then (constant angle, 0), then
  * (pair angle, 0) for every qubit pair j < l in row order. A tile pass's record is followed by the records
  * (and matrices) of its member blocks in the order the pass applies them;
- * they carry the pass's index. *n_blocks (records) and *mats_len (complex
+ * they carry the pass's index. (The members of a tensor-core tile pass: dense
+ * blocks of up to 7 qubits, block-diagonal in at most two outside the tile.)
+ * *n_blocks (records) and *mats_len (complex
  * entries) receive the totals.
  */
 qs_status qs_plan(int n, const qs_gate *gates, size_t n_gates, uint64_t flags, const qs_opts *opts,

@@ -311,7 +311,7 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
     return fail(QS_EUNSUPPORTED, "qs_apply_circuit: global bits (opts.n_global) need a sharded runner; "
                                  "qs_plan plans their exchanges");
   DeviceGuard dg(st->device);
-  const bool by_rules = (flags & QS_PGO_RULES) && !(flags & QS_PGO_MEASURED);
+  const uint64_t asked = flags;
   // fold the timings of an earlier profiled call that has finished
   fold_records(st, false);
   if (flags & QS_PGO_MEASURED) {
@@ -328,12 +328,7 @@ qs_status qs_apply_circuit(qs_state *st, const qs_gate *gates, size_t n_gates, u
   const bool c128 = st->dtype == QS_C128;
   const int ab = amp_bytes(st);
   const bool prof = flags & QS_PROFILE;
-  // tensor-core tile passes where the rules choose the kernels (explicit flags
-  // run the blocks they ask for): not where each block is timed (their times
-  // are what the other activators learn from), nor where the options ask for
-  // a kernel
-  bool tiles = by_rules && !c128 && !prof && st->n > kTcTileBits && (flags & QS_TC) && o.threads == 0 &&
-               o.tc_exchange == 0 && o.tc_precision == 0;
+  bool tiles = tc_tiles_apply(st->n, c128, asked, flags, o);
   std::vector<Block> plan;
   PlanStats stats;
   std::string err;
@@ -670,13 +665,15 @@ qs_status qs_plan(int n, const qs_gate *gates, size_t n_gates, uint64_t flags, c
   qs_opts o;
   if (opts) o = *opts;
   else qs_default_opts(&o);
+  const uint64_t asked = flags;
   if (flags & QS_PGO_RULES) flags = rules_select(n, false, gates, n_gates, o, flags);
   std::vector<Block> plan;
   PlanStats stats;
   std::string err;
   int8_t perm[QS_MAX_QUBITS];
   std::memcpy(perm, perm_inout, n);
-  qs_status s = build_plan(n, gates, n_gates, flags, o, perm, plan, stats, err);
+  qs_status s = build_plan(n, gates, n_gates, flags, o, perm, plan, stats, err, false, true, false,
+                           tc_tiles_apply(n, false, asked, flags, o));
   if (s != QS_OK) return fail(s, "qs_plan: " + err);
   std::memcpy(perm_inout, perm, n);
   size_t mlen = 0, nr = 0;
@@ -699,7 +696,7 @@ qs_status qs_plan(int n, const qs_gate *gates, size_t n_gates, uint64_t flags, c
   };
   for (size_t i = 0; i < plan.size(); i++) {
     emit(plan[i], (int)i);
-    for (const Block &m : plan[i].sub) emit(m, (int)i);  // a tile pass's members, in order
+    for (const Block &m : plan[i].sub) emit(plan[i].tc ? tile_member_block(m) : m, (int)i);  // a pass's members, in order
   }
   if (n_blocks) *n_blocks = nr;
   if (mats_len) *mats_len = mlen;

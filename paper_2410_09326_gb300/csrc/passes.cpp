@@ -1023,6 +1023,41 @@ void fill_record(const Block &b, int index, int n, int amp_bytes, qs_block_recor
   r.ms = -1;
 }
 
+bool tc_tiles_apply(int n, bool c128, uint64_t flags, uint64_t chosen, const qs_opts &o) {
+  return (flags & QS_PGO_RULES) && !(flags & (QS_PGO_MEASURED | QS_PROFILE)) && (chosen & QS_TC) && !c128 &&
+         n > kTcTileBits && o.threads == 0 && o.tc_exchange == 0 && o.tc_precision == 0 && o.n_global == 0;
+}
+
+Block tile_member_block(const Block &m) {
+  // the qubits that some gate acts on, ascending: its targets without the
+  // identity's, and the bits outside the tile
+  auto qubit = [&](int at) { return at >= 0 ? m.q[at] : m.sel[-1 - at]; };
+  uint64_t mask = 0;
+  for (const Block::Member &g : m.gates)
+    for (int j = 0; j < g.nq; j++) mask |= 1ull << qubit(g.at[j]);
+  Block out;
+  out.kind = BK_DENSE;
+  out.tc = true;
+  out.n_gates = m.n_gates;
+  for (int q = 0; q < 64; q++)
+    if ((mask >> q) & 1) out.q[out.k++] = q;
+  Product M(out.k);
+  size_t at = 0;
+  for (const Block::Member &g : m.gates) {
+    const size_t entries = (size_t)1 << (2 * g.nq);
+    const std::vector<cd> G(m.mat.begin() + (long)at, m.mat.begin() + (long)(at + entries));
+    int pos[3] = {0, 0, 0};
+    for (int j = 0; j < g.nq; j++) pos[j] = pos_of(out.q, out.k, qubit(g.at[j]));
+    left_multiply(M, G, pos, g.nq);
+    at += entries;
+  }
+  const int d = 1 << out.k;
+  out.mat.resize((size_t)d * d);
+  for (int r = 0; r < d; r++)
+    for (int c = 0; c < d; c++) out.mat[(size_t)r * d + c] = M.at(r, c);
+  return out;
+}
+
 double block_bytes(const Block &b, int n, int amp_bytes) {
   double amps = std::ldexp(1.0, n - b.nctrl);
   if (b.kind == BK_PERMUTE || b.kind == BK_GLOBAL) amps = std::ldexp(1.0, n - 1);

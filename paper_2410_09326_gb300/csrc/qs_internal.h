@@ -162,6 +162,16 @@ int tile_k_of(const qs_opts &o);
 
 double block_bytes(const Block &b, int n, int amp_bytes);
 
+// Whether a call under these options may run as tensor-core tile passes: where
+// the rules choose the kernels (explicit flags run the blocks they ask for) and
+// each block is not timed (the times are what the other activators learn from),
+// unless the options ask for a kernel. flags: as given; chosen: by the rules.
+bool tc_tiles_apply(int n, bool c128, uint64_t flags, uint64_t chosen, const qs_opts &o);
+
+// A member of a tensor-core tile pass as the block it is of the whole state:
+// its product over its qubits inside and outside the tile (up to seven).
+Block tile_member_block(const Block &member);
+
 // The public record of a planned block (passes.cpp).
 void fill_record(const Block &b, int index, int n, int amp_bytes, qs_block_record &r);
 

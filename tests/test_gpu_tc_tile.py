@@ -88,6 +88,22 @@ def test_errors_of_many_blocks_do_not_add_up():
     assert np.linalg.norm(got - want) <= 1.2e-6
 
 
+@pytest.mark.parametrize("n", [13, 14, 17, 23])
+def test_the_plan_is_what_runs(n):
+    gates = _layers(n, 4, n, ["cx", "cp", "ccx", "swap"])
+    st = qs.qs_alloc_state(n, qs.QS_C64)
+    try:
+        qs.qs_apply_circuit(st, qs.gates_to_array(gates), FLAGS)
+        ran = qs.qs_profile(st)[1]
+    finally:
+        qs.qs_free_state(st)
+    plan = qs.qs_plan(n, qs.gates_to_array(gates), FLAGS)[0]
+    assert any(r.kind == 3 for r in plan) == (n > 13)
+    plan = [r for i, r in enumerate(plan) if i == 0 or r.index != plan[i - 1].index]  # without the passes' members
+    assert [(r.kind, r.k, r.tc, r.n_gates, r.cmask, list(r.qubits)) for r in ran] == \
+        [(r.kind, r.k, r.tc, r.n_gates, r.cmask, list(r.qubits)) for r in plan]
+
+
 def test_every_block_controlled_from_outside_the_tile():
     """Blocks that only act where the highest bits are 1: tiles without work are left as they are."""
     n, top = 15, [13, 14]
