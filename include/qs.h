@@ -126,9 +126,9 @@ typedef struct {
   int fuse_lookahead;   /* fusion: where a gate could join several blocks or open a new one,
                            each choice is followed by this many gates of first-fit placement
                            and the one leaving the fewest blocks is taken; 0 = first fit
-                           (qs_default_opts: 60). Narrow states (below 23 qubits, complex128 below
-                           22) take first fit outside batches: the search would cost more host
-                           time than the blocks it saves */
+                           (qs_default_opts: 60). The default is searched where the blocks it
+                           saves are worth its host time: from 23 qubits on (complex128: 22) and
+                           in batches; any other horizon at every width */
   int no_shuffles;      /* 1: CUDA-core blocks whose targets cover bits 1, 2, 3 (bit 0 free) keep
                            the thread-per-group kernel instead of warp-wide loads and shuffles (c64) */
   int tc_exchange;      /* 4- to 6-target tensor-core blocks (FP16 halves): the thread-per-group

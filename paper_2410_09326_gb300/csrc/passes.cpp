@@ -874,9 +874,11 @@ qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<
     // passes take five times as long and pay from 22 on), or where a plan is
     // run again and again (a batch). Without free joins they cost 5 us per
     // gate and sometimes save a few blocks more at 6 targets (98 instead of
-    // 107 for the 30-qubit random circuit): from 27 qubits on (25).
+    // 107 for the 30-qubit random circuit): from 27 qubits on (25). A caller
+    // that asks for another horizon than the default gets all of it.
     const int wide = n + (c128 ? 1 : 0);
-    const bool search = opts.fuse_lookahead > 0 && (wide >= kSearchBits || repeated);
+    const bool asked = opts.fuse_lookahead > 0 && opts.fuse_lookahead != kLookahead;
+    const bool search = opts.fuse_lookahead > 0 && (wide >= kSearchBits || repeated || asked);
     first_fit(groups);
     // (a circuit of one block gains nothing from a tile: three targets at 26
     // qubits 341 us with the call's host time, 323 us by itself, at 16 qubits
@@ -886,7 +888,7 @@ qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<
       // has many gates (all pairs of 26 qubits in one diagonal run, 325 gates,
       // lost 0.5 ms to them). Layered circuits have 11 to 14 gates to a block.
       const double block_gates = std::ldexp(16.0, n - (n < kPassSearchBits ? kSearchBits : kPassSearchBits));
-      const bool roll_outs = search && (double)all.size() <= block_gates * (double)groups.size();
+      const bool roll_outs = asked || (search && (double)all.size() <= block_gates * (double)groups.size());
       tiled_cost = tc_tile_passes(n, pg, all, K, roll_outs, passes);
       // not searched where no search (it saves one block in six) would change the choice
       tiled_tc = tiled_cost < (search ? 0.8 : 1.0) * (double)groups.size();
@@ -904,7 +906,7 @@ qs_status plan_segment(int n, const std::vector<qs_gate> &pg, const std::vector<
       const Variant variants[] = {{0, 0, false},          {L, 6, true},       {L, 12, true},
                                   {L + L / 3, 6, true},   {L, 6, false},      {L, 12, false},
                                   {L + L / 3, 6, false},  {L + L / 3, 12, false}, {L + 2 * L / 3, 6, false}};
-      const size_t count = n + (c128 ? 2 : 0) >= kFullSearchBits ? 9 : 4;
+      const size_t count = n + (c128 ? 2 : 0) >= kFullSearchBits || asked ? 9 : 4;
       std::vector<std::vector<Pending>> alt(count);
       auto one = [&](size_t v) {
         if (v == 0) alt[0] = groups;

@@ -723,3 +723,27 @@ def test_lookahead_fusion_never_adds_blocks_and_saves_them_on_layered_circuits()
         arr = qs.gates_to_array(c[name][1])
         flags = qs.QS_VSWAP | qs.QS_FUSE | qs.QS_FUSE_K(5) | qs.QS_DIAG
         assert len(qs.qs_plan(30, arr, flags)[0]) <= len(qs.qs_plan(30, arr, flags, opts=first)[0])
+
+
+@pytest.mark.parametrize("n", [16, 20, 22])
+def test_a_fusion_horizon_that_was_set_is_searched_on_narrow_states(n):
+    """The default is not (first fit costs less than the search saves there); any other horizon is what a caller
+    asked for."""
+    rng = cg.SplitMix64(7)
+    gates = []
+    for _ in range(12):
+        gates += [("u3", [q], [rng.uniform(0, 6.28) for _ in range(3)]) for q in range(n)]
+        q = list(range(n))
+        for i in range(n - 1, 0, -1):
+            j = rng.randint(i + 1)
+            q[i], q[j] = q[j], q[i]
+        gates += [("cx", [q[2 * i], q[2 * i + 1]]) for i in range(n // 2)]
+    arr = qs.gates_to_array(gates)
+    flags = qs.QS_VSWAP | qs.QS_FUSE | qs.QS_FUSE_K(5) | qs.QS_DIAG
+    blocks = {}
+    for horizon in (0, 60, 61):
+        opts = qs.qs_default_opts()
+        opts.fuse_lookahead = horizon
+        blocks[horizon] = len(qs.qs_plan(n, arr, flags, opts=opts)[0])
+    assert blocks[60] == blocks[0] == len(qs.qs_plan(n, arr, flags)[0])
+    assert blocks[61] <= 0.9 * blocks[0]
