@@ -12,10 +12,13 @@ import paper_2410_09326_gb300 as qs
 pytestmark = pytest.mark.gpu
 
 
-# errors per block: 4e-7 (FP16 halves, FP32 sums) and 1e-16 (digit planes); 1203 of them add up at most
-@pytest.mark.parametrize("dtype,k,bound", [(qs.QS_C64, 4, 4e-7), (qs.QS_C64, 5, 4e-7), (qs.QS_C64, 6, 4e-7),
-                                           (qs.QS_C128, 4, 1e-16), (qs.QS_C128, 5, 1e-16)])
-def test_many_blocks(dtype, k, bound):
+# a block's error in a direction of its own, and what truncation takes off the norm, of the same sign in every
+# block (below the spacing of FP32 numbers at the factor that puts the norm right): 1.2e-7 and 2.4e-8 with FP16
+# halves, 1e-16 and none with digit planes; the FP64 oracle's own 1e-16 for each of 13 to 17 gates of a block
+@pytest.mark.parametrize("dtype,k,own,common", [
+    (qs.QS_C64, 4, 1.2e-7, 2.4e-8), (qs.QS_C64, 5, 1.2e-7, 2.4e-8), (qs.QS_C64, 6, 1.2e-7, 2.4e-8),
+    (qs.QS_C128, 4, 4e-16, 0), (qs.QS_C128, 5, 4e-16, 0)])
+def test_many_blocks(dtype, k, own, common):
     n, blocks = 2 * k - 1, 1203  # two sets of k qubits that share one: blocks alternate and cannot merge
     r = random.Random(k)
     gates = []
@@ -32,4 +35,5 @@ def test_many_blocks(dtype, k, bound):
     finally:
         qs.qs_free_state(st)
     want, _ = oracle.simulate(cg.to_qasm(n, gates))
-    assert np.linalg.norm(got - want) <= bound * blocks
+    e = np.linalg.norm(got - want)
+    assert e <= 1.5 * (own * blocks ** 0.5 + common * blocks)
