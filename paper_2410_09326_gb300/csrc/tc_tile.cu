@@ -124,7 +124,8 @@ __device__ __forceinline__ NormFix norm_fix(float nin, float nout) {
   const uint32_t scb = norm_scale(nin);  // again: it need not stay in a register
   const float sc = __uint_as_float(scb);
   // an exact difference of near numbers: approximate quotients and roots do for the rest
-  const float r = nout > 0.f ? __fdividef(fmaf(nin * sc, sc * (kB * kB), -nout), nout) : 0.f;
+  // (-1 where nin has underflowed: the row becomes zero)
+  const float r = nout > 0.f ? fmaxf(__fdividef(fmaf(nin * sc, sc * (kB * kB), -nout), nout), -1.f) : 0.f;
   float q;
   asm("sqrt.approx.f32 %0, %1;" : "=f"(q) : "f"(1.f + r));
   const uint32_t d = __float_as_uint(__fdividef(r, 1.f + q));

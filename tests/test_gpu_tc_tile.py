@@ -94,6 +94,23 @@ def test_errors_of_many_blocks_do_not_add_up():
     assert np.linalg.norm(got - want) <= 1.2e-6
 
 
+@pytest.mark.parametrize("size", [1e-17, 1e-20, 1e-22, 1e-23, 1e-24, 1e-26, 1e-30, 1e-36, 1e-40])
+def test_rows_whose_norm_underflows(size):
+    """What cancellations leave behind: amplitudes whose squares are subnormal or zero in FP32. They may come out as
+    zero, never larger than they were, and never as NaN."""
+    n = 14
+    gates = _layers(11, 3, 3, ["cx"])
+    init = _random_state(n, 4).reshape(8, 1 << 11)
+    init[1:] *= size
+    init = init.astype(np.complex64)
+    got, recs = _run(n, gates, init.reshape(-1))
+    got = got.reshape(8, 1 << 11)
+    assert any(r.kind == 3 for r in recs) and np.isfinite(got).all()
+    assert np.abs(np.linalg.norm(got[0]) / np.linalg.norm(init[0].astype(np.complex128)) - 1) <= 1e-6
+    for i in range(1, 8):
+        assert np.linalg.norm(got[i]) <= 1.01 * np.linalg.norm(init[i].astype(np.complex128)) + 1e-44
+
+
 def test_products_of_a_split_pass():
     """More blocks than a launch takes, most of them with two bits outside the tile that pick one of four products:
     the second launch's products follow the first's."""
