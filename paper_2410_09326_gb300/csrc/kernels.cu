@@ -724,10 +724,16 @@ cudaError_t launch_permute(void *amps, int n, bool c128, int qa, int qb, cudaStr
 
 cudaError_t launch_bit_swaps(void *amps, int n, bool c128, const std::vector<std::pair<int, int>> &swaps,
                              cudaStream_t s) {
-  // one exchange moves half the state; two of them moved a 16 MiB state in
-  // 7.8 us as two launches, 12.4 us together, a 2 GiB one in 1140 and 943
+  // One exchange moves half the state, so that two by themselves move no more
+  // than both together. Those of a bit within a 128-byte run move whole lines
+  // for half of it: two of these together from 128 MiB on (bits 0, 3 and 1, 2:
+  // 24 qubits 409 -> 394 us, 28 qubits 5.76 -> 5.35 ms, complex128 0.90; of
+  // bits above 4: 28 qubits 5.14 by themselves, 5.43 together, complex128 up
+  // to 1.29 times as long; times with the distance of two states behind).
   const size_t bytes = (size_t)(c128 ? 16 : 8) << n;
-  if (swaps.size() < 2 || (swaps.size() == 2 && bytes < (128ull << 20))) {
+  const int low = c128 ? 3 : 4, full = c128 ? 6 : 7;
+  const bool lines = std::all_of(swaps.begin(), swaps.end(), [&](const std::pair<int, int> &x) { return x.first < low; });
+  if (swaps.size() < 2 || (swaps.size() == 2 && !(lines && bytes >= (128ull << 20)))) {
     for (const auto &x : swaps) {
       cudaError_t e = launch_permute(amps, n, c128, x.first, x.second, s);
       if (e != cudaSuccess) return e;
@@ -740,7 +746,6 @@ cudaError_t launch_bit_swaps(void *amps, int n, bool c128, const std::vector<std
     to[x.first] = x.second;
     to[x.second] = x.first;
   }
-  const int low = c128 ? 3 : 4, full = c128 ? 6 : 7;
   uint64_t tile = 0;
   int t = 0;
   auto take = [&](int q) {
