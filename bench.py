@@ -352,22 +352,24 @@ def run_ours(args):
 
 # DRAM bytes (read + write) per launch of a kernel, from one ncu capture of
 # it at n = 26 scaled to n = 30 by the amplitudes processed (x16), with the
-# SHA-256 prefix of the source file the captured kernel was built from: once
-# that file changes the capture no longer describes the kernel and the
-# traffic is reported as null.
-TRAFFIC_PER_LAUNCH = {"k_dense_k5_tcx": (16.18e9, "tc16x.cu", "91553d61b5d5d04b"),
-                      "k_dense_k6_tcx": (16.17e9, "tc16x.cu", "91553d61b5d5d04b"),
-                      "k_dense_k4_tc": (16.17e9, "tc16.cu", "82ff16b73b52bb19")}
+# SHA-256 prefix of the source file the captured kernel was built from and the
+# headers it shares: once one of them changes the capture no longer describes
+# the kernel and the traffic is reported as null.
+TRAFFIC_PER_LAUNCH = {"k_dense_k5_tcx": (16.17e9, "tc16x.cu", "4d8f120d9bcd98ec"),
+                      "k_dense_k6_tcx": (16.17e9, "tc16x.cu", "4d8f120d9bcd98ec"),
+                      "k_dense_k4_tc": (16.17e9, "tc16.cu", "4385cfef58a19d72")}
 
 
 def _source_digest(fname):
     import hashlib
-    path = os.path.join(ROOT, "paper_2410_09326_gb300", "csrc", fname)
+    h = hashlib.sha256()
     try:
-        with open(path, "rb") as f:
-            return hashlib.sha256(f.read()).hexdigest()[:16]
+        for name in (fname, "tc16_common.cuh", "tc_common.cuh", "kernels_common.cuh"):
+            with open(os.path.join(ROOT, "paper_2410_09326_gb300", "csrc", name), "rb") as f:
+                h.update(f.read())
     except OSError:
         return None
+    return h.hexdigest()[:16]
 
 
 def traffic_per_launch(kernel):

@@ -652,9 +652,10 @@ qs_status tile_plan(int n, const std::vector<qs_gate> &pg, const std::vector<int
 }
 
 // Cost of a tile pass of b blocks, in launches of a single block of up to five
-// targets. Measured 0.45 + 0.4 b: at 27 qubits, where a block is an HBM pass,
-// 80 for the 30-qubit random circuit's 45 passes with 151 blocks (125 blocks
-// one by one), and as much at 19 qubits, where launches and latency count.
+// targets: 0.45 + 0.4 b, fitted to passes at 27 qubits, where a block is an HBM
+// pass, and as good at 19 qubits, where launches and latency count. (It puts
+// the 39 passes of the 30-qubit random circuit, 116 blocks, at 64; they take
+// 165 ms, the circuit's 126 blocks one by one 339.)
 double tc_tile_cost(size_t b) { return 0.45 + 0.4 * (double)b; }
 
 // Tensor-core tile passes (tc_tile.cu): gates grouped as in tile_plan into

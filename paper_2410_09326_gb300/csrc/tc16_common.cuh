@@ -99,7 +99,7 @@ __device__ __forceinline__ void operand_halves(int odd, float re, float im, uint
 }
 
 // The lane-exchange kernels (tc16x.cu) for a block the planner marked for
-// them (b.tc_xg); B must have been built in slot order (tc16_build_b does).
+// them (b.tc_xg); B must be in slot order (operands.cu makes it so).
 cudaError_t run_dense_tc16x(float2 *a, int n, const Block &b, const void *dev_b, int *err, cudaStream_t s,
                             LaunchShape *shape);
 

@@ -5,7 +5,7 @@
 // element (warp shuffles; lane/register exchanges of the loads, where lane
 // bit 0 takes no part, by the staging copies' placement) until each lane
 // holds one whole group; B is built
-// in the same "slot" order (tc16_build_b). The host layout (which bits sit on
+// in the same "slot" order (operands.cu). The host layout (which bits sit on
 // lanes and registers, which exchanges run) is tc_exchange_layout below; the
 // planner picks these kernels where tc_exchange_pays.
 #include <algorithm>

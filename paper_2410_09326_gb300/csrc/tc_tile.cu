@@ -13,17 +13,16 @@
 // Per block, a thread reads its group from shared memory, scales and splits it
 // into FP16 halves as tc16.cu does, writes them to its lane of tensor memory
 // (the MMA takes A from there: nothing but the tile and B is in shared
-// memory), and after the MMAs rescales its row of the product to the group's
-// norm and writes it back in place. The three products share one accumulator,
+// memory), and after the MMAs brings its row of the product back to the
+// group's norm (norm_fix) and writes it in place. The three products share one accumulator,
 // the small ones first, so that the accumulation's truncation costs no more
 // than with an accumulator of their own. B of the next block (16 KB, hi and
 // lo) is copied in as soon as this block's MMAs have read theirs.
 //
-// At 26 qubits a pass of four blocks takes 328 us, three 301 us, one block by
+// At 26 qubits a pass of four blocks takes 321 us, three 274 us, one block by
 // itself 172 us (one HBM pass: 160 us); the 30-qubit 30-layer random circuit
-// 335 -> 172 ms. Bound by the serial chain of a block (5,600 cycles at four
-// CTAs per SM, 4,200 alone), the issue slots at 44% and the shared-memory pipe
-// at 53%. 13-bit tiles in two CTAs of 256 threads were 8% slower at 27 qubits,
+// 339 ms as single blocks, 165 to 169 on tile passes. Bound by the serial chain
+// of a block, the issue slots at 47% and the shared-memory pipe at 52%. 13-bit tiles in two CTAs of 256 threads were 8% slower at 27 qubits,
 // two accumulations of the large products 10% (their error 5% less).
 //
 // Shared memory holds amplitude i at byte address i * 8 with its 16-byte
