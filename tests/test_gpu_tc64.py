@@ -153,11 +153,14 @@ def test_small_rotations_keep_their_small_amplitudes(flags):
     assert (np.abs(got - want) <= 3 * 2.0 ** (6 - 53) * np.abs(want)).all()
 
 
-@pytest.mark.parametrize("targets", [[0, 1, 2, 3], [0, 1, 2, 3, 4], [1, 4, 6, 9], [2, 3, 7, 8, 11]])
+# part of a tile, one tile, tiles that three CTAs loop over
+@pytest.mark.parametrize("n,targets,ctas", [
+    (7, [0, 1, 2, 3], 0), (8, [0, 2, 4, 5, 7], 0), (11, [0, 1, 2, 3], 0), (12, [2, 3, 7, 8, 11], 0),
+    (15, [1, 4, 6, 9], 3), (16, [0, 1, 2, 3, 4], 3)])
 @pytest.mark.parametrize("tiny", [0.0, 1e-7])
-def test_groups_of_very_different_amplitudes_take_fp64(targets, tiny):
+def test_groups_of_very_different_amplitudes_take_fp64(n, targets, ctas, tiny):
     """A matrix that mixes one qubit and moves the others about keeps small amplitudes apart from large ones."""
-    n, k, r = 12, len(targets), random.Random(len(targets))
+    k = len(targets)
     gates = [("u3", [targets[0]], [1.1, 0.3, 0.7])]
     gates += [("cx", [a, b], []) for _ in range(2) for a, b in zip(targets, targets[1:] + targets[:1])]
     if tiny:  # weights far below 1 between the halves of another qubit
@@ -178,8 +181,10 @@ def test_groups_of_very_different_amplitudes_take_fp64(targets, tiny):
     at = low[:, None] + np.array([sum(((s >> j) & 1) << q for j, q in enumerate(targets)) for s in range(1 << k)])
     x = np.zeros(1 << n, dtype=np.complex128)
     x[at] = y
-    got, recs, width = _run(n, gates, x)
-    assert [(q.k, q.tc) for q in recs] == [(k, 1)]
+    opts = qs.qs_default_opts()
+    opts.tc_max_ctas = ctas
+    got, recs, width = _run(n, gates, x, opts)
+    assert [(q.k, q.tc) for q in recs] == [(k, 1)] and (not ctas or recs[0].tiles > 2 * recs[0].ctas)
     _, (mat,), _ = qs.qs_plan(n, gates, qs.QS_FUSE | qs.QS_FUSE_K(width))
     m = mat.astype(np.clongdouble)
     want = np.stack([(m * v).sum(1) for v in y.astype(np.clongdouble)])
