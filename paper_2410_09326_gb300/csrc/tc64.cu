@@ -36,10 +36,10 @@
 // (small entries). So groups are looked at where the matrix has entries below
 // 2^-20: if an amplitude lies below 2^-20 of the largest (zeros count where
 // small entries are not zero), the group takes the FP64 mat-vec (exact_groups).
-// The look costs 3% (24 qubits, 10 layers, median of 60 random circuits 8.39 ->
-// 8.61 ms); a block whose groups all span more, as early layers with an angle
-// near a multiple of pi leave them, costs an FP64 pass: 3 of the 60 took 1.25
-// to 1.9 times as long (7 with 2^-16), the mean 8.43 -> 8.85 ms.
+// The look costs 1% (24 qubits, 10 layers, median of 30 random circuits 8.41 ->
+// 8.52 ms); a block whose groups all span more, as early layers with an angle
+// near a multiple of pi leave them, costs an FP64 pass: of 60 such circuits
+// three took 1.25 to 1.9 times as long (with 2^-16, seven).
 //
 // Measured at n = 25 (1 GiB read and written), FP64 kernel -> this one: 5
 // targets 6930 -> 430 us, 4 targets 4080 -> 330 us (3.2 TB/s); bits 0..4:
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(Tc64<K>::NT, Tc64<K>::CTAS)
   unsigned char *sB = smem + kDigitsA * C::A_BYTES;
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ uint32_t tmem_slot;
-  __shared__ uint32_t red[2][NT];
+  __shared__ uint32_t red[NT];
   __shared__ uint32_t exact_rows[4];
 
   const int tid = threadIdx.x;
@@ -247,24 +247,22 @@ __global__ void __launch_bounds__(Tc64<K>::NT, Tc64<K>::CTAS)
 
   for (; tile < p.n_tiles; tile += gridDim.x) {
     // the group's exponent: the largest high word without its sign; and that
-    // of its smallest amplitude (check 1: of the nonzero ones)
-    uint32_t mx = 0, mn = 0x7fffffffu;
+    // of its smallest amplitude (check 1: of the nonzero ones), both in one word
+    uint32_t mx = 0, mn = 0xffffffffu;
+    const uint32_t skip_zero = check == 1;  // 0 - 1 is the largest
 #pragma unroll
     for (int u = 0; u < 8; u++) {
       const uint32_t m = max((uint32_t)__double2hiint(v[u].x) & 0x7fffffffu, (uint32_t)__double2hiint(v[u].y) & 0x7fffffffu);
       mx = max(mx, m);
-      mn = min(mn, check == 1 && m == 0 ? 0x7fffffffu : m);
+      mn = min(mn, m - skip_zero);
     }
-    red[0][tid] = mx;
-    if (check) red[1][tid] = mn;
+    uint32_t span = (mx >> 20 << 16) | (0xffffu - (mn >> 20));
+    red[tid] = span;
     if (!__syncthreads_and(ok)) break;  // a wait of the last tile ran out
 #pragma unroll
-    for (int o = 1; o < C::TPR; o++) {
-      mx = max(mx, red[0][(tid + o * 128) % NT]);
-      if (check) mn = min(mn, red[1][(tid + o * 128) % NT]);
-    }
-    const int gexp = max((int)(mx >> 20), 1);  // subnormals count from exponent 1
-    const bool exact = check && gexp < 2047 && gexp - (int)(mn >> 20) > kDigitSpan;
+    for (int o = 1; o < C::TPR; o++) span = __vmaxu2(span, red[(tid + o * 128) % NT]);
+    const int gexp = max((int)(span >> 16), 1);  // subnormals count from exponent 1
+    const bool exact = check && gexp < 2047 && gexp - (int)(0xffffu - (span & 0xffffu)) > kDigitSpan;
 #pragma unroll
     for (int hh = 0; hh < 2; hh++) {
       uint64_t f[8];
@@ -274,6 +272,10 @@ __global__ void __launch_bounds__(Tc64<K>::NT, Tc64<K>::CTAS)
         f[2 * u + 1] = to_digits(v[4 * hh + u].y, gexp);
       }
       store_digits<0, K>(f, sA, row_off + (uint32_t)(hh * C::TPR + q) * C::LBO);
+    }
+    if (check && tid < 128) {  // warps 0..3 have every row once
+      const uint32_t rows = __ballot_sync(0xffffffffu, exact);
+      if ((tid & 31) == 0) exact_rows[warp] = rows;
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;");
@@ -338,10 +340,7 @@ __global__ void __launch_bounds__(Tc64<K>::NT, Tc64<K>::CTAS)
       }
     }
     phase ^= 1;
-    if (check && __syncthreads_or(exact)) {
-      const uint32_t rows = __ballot_sync(0xffffffffu, exact);
-      if (tid < 128 && (tid & 31) == 0) exact_rows[warp] = rows;
-      __syncthreads();
+    if (check && (exact_rows[0] | exact_rows[1] | exact_rows[2] | exact_rows[3])) {
       exact_groups<K>(a, reinterpret_cast<const double2 *>(bmat + C::B_BYTES / 16), p, tile, exact_rows);
     }
   }
